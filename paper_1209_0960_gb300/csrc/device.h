@@ -172,13 +172,26 @@ __host__ __device__ inline bool bi_continue(BiScalars& b) {
 // the pass counters count finished items over all launches.
 struct SweepPass {
     int32_t r0, r1;   // rows of the pass's colour (smoothing order)
-    int32_t jmax;     // neighbours at positions >= jmax are taken as zero
+    int32_t jmax;     // neighbours at positions >= jmax are taken as zero (rows not split)
     int32_t first;    // 1: colour 0 from a zero guess, x = b / A_ii
+    int32_t part;     // the entries of a split level's rows it reads (RowPart)
     int32_t tiles;    // items of the pass
     int32_t item0;    // index of its first item
 };
 
 constexpr int kSweepMaxPasses = 64;
+
+// Entries of a split level's rows that a colour pass of symmetric
+// Gauss-Seidel reads, with s_i = b_i - (lower part)_i x kept from the forward
+// pass over the row:
+//   kPartLower  forward from a zero guess (later colours still zero):
+//               s = b - L x, x = s / A_ii
+//   kPartUpper  backward: the lower neighbours have not changed since the
+//               forward pass, so x = (s - U x) / A_ii
+//   kPartBoth   forward from a non-zero guess: s = b - L x, x = (s - U x) / A_ii
+// and after the backward sweep the residual is (b - s) - L x, because the last
+// update made s = A_ii x + U x.
+enum RowPart : int32_t { kPartLower = 0, kPartUpper = 1, kPartBoth = 2 };
 
 struct SweepPlan {
     int32_t rows = 0;                        // rows per item
@@ -217,6 +230,7 @@ struct DevLevel {
     int32_t n_coarse = 0;
     std::vector<int32_t> cptr;        // host copy: first row of each colour, [ncolours+1]
     std::vector<int64_t> cnnz;        // host copy: off-diagonal entries of each colour block
+    std::vector<int64_t> clow;        // split levels: those towards earlier colours
     int32_t lpr = 0;                  // lanes per row of the row kernels: 0 = the fine
                                       // level's kernels (one row per thread, slices staged
                                       // in shared memory, tiles within kMaxStageBytes), else
@@ -229,6 +243,12 @@ struct DevLevel {
                                       // aggregates of at most 32 rows of colour 1)
     int32_t* err = nullptr;           // device status word for kernel-side errors (timeouts)
     uint16_t* rlen = nullptr;         // [n] off-diagonal entries per row
+    // split rows (coarse levels of three or more colours): the entries of a
+    // row towards earlier colours (rlow of them, the lower part) fill its slots
+    // 0, 1, ... and those towards later colours (the upper part) the slots
+    // W - 1, W - 2, ..., so a pass that needs one part reads whole lines of it
+    bool split = false;
+    uint16_t* rlow = nullptr;         // [n] entries towards earlier colours (split levels)
     int32_t* scol = nullptr;          // [padded] permuted column indices
     double* sval = nullptr;           // [padded]
     // sliced layout with per-slice widths, for the staged kernels on levels
@@ -420,6 +440,7 @@ struct VArgs {
     int32_t r0 = 0, r1 = 0, jmax = 0, n = 0, nc = 0, width = 0, ld = 0;
     int64_t sw = 0, nslices = 0, cap = 0;
     const uint16_t* rlen = nullptr;
+    const uint16_t* rlow = nullptr;   // split levels: entries towards earlier colours
     const int32_t* scol = nullptr;
     const int32_t* idx = nullptr;     // aggregate map, or restriction list pointers
     const int32_t* idx2 = nullptr;    // restriction list rows
@@ -478,8 +499,11 @@ void launch_first(const DevLevel& L, const double* b, double* x, double* bc_zero
                   cudaStream_t s);
 void launch_first32(const DevLevel& L, const float* b, float* x, float* bc_zero, int nc,
                     cudaStream_t s);
-void launch_pass(const DevLevel& L, int col, int jmax, const double* b, double* x, cudaStream_t s);
-void launch_pass32(const DevLevel& L, int col, int jmax, const float* b, float* x, cudaStream_t s);
+// part: which part of a split level's rows the pass reads (ignored elsewhere)
+void launch_pass(const DevLevel& L, int col, int jmax, RowPart part, const double* b, double* x,
+                 cudaStream_t s);
+void launch_pass32(const DevLevel& L, int col, int jmax, RowPart part, const float* b, float* x,
+                   cudaStream_t s);
 // fine level of the float32 V-cycle: the first pass forms b = r / s from the
 // float64 residual (isq = 1/s), and the last pass over each colour also
 // writes z = x / s in float64 (the V-cycle's output)
@@ -559,8 +583,9 @@ void galerkin_device(const DevCsr& A, const HostCsr& Ah, const AggResult& agg, D
 
 // Build the smoothing-order device level from the original-order device
 // matrix A and the permutation perm (original -> new position).
+// split: store the rows split by colour (see DevLevel::split).
 void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<int32_t>& perm,
-                        DevArena& arena, DevLevel& L, cudaStream_t s);
+                        bool split, DevArena& arena, DevLevel& L, cudaStream_t s);
 
 // Decoupled aggregation (Alg. 4) on the device: the rows of A (original
 // order) split into consecutive tiles of p.aggregation_tile rows, one warp per

@@ -402,6 +402,199 @@ struct ResidualBody {
 };
 
 // ---------------------------------------------------------------------------
+// Split levels (DevLevel::split): a pass reads the part of the rows it needs.
+//
+// A symmetric sweep that reads whole rows in every pass streams the matrix
+// five times per V-cycle and level (forward, backward, residual, forward,
+// backward).  Keeping s = b - L x of the forward pass makes it three times
+// (see RowPart): the backward passes read the upper parts only, the forward
+// passes from a zero guess and the residual the lower parts only.  The passes
+// of a coarse level are bound by their gathers of x and by the float64 pipe,
+// both of which shrink with the entries.
+// ---------------------------------------------------------------------------
+
+// entries per lane of one batch of a row part
+template <int LPR>
+__host__ __device__ constexpr int part_unroll() { return LPR <= 2 ? 8 : LPR == 4 ? 4 : 2; }
+
+template <int LPR, typename T>
+struct PartBatch {
+    static constexpr int U = part_unroll<LPR>();
+    int j[U];
+    T a[U];
+    // entries lane + (it U + u) LPR of the part: slots 0, 1, ... of the lower
+    // part, last, last - 1, ... of the upper part; j = -1 past its end
+    template <bool UPPER>
+    __device__ __forceinline__ void load(int it, int64_t base, int cnt, int last, int lane,
+                                         const int32_t* __restrict__ scol,
+                                         const T* __restrict__ sval, int nrows, int32_t* err) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = lane + (it * U + u) * LPR;
+            const bool in = t < cnt;
+            const int64_t e = base + 32 * (int64_t)(in ? (UPPER ? last - t : t) : 0);
+            j[u] = in ? scol[e] : -1;
+            a[u] = in ? sval[e] : T(0);
+            if (kChecks && in && !index_ok(j[u], nrows, err)) j[u] = -1;
+        }
+    }
+};
+
+// acc - sum of the part's entries of this lane times the neighbour values;
+// B holds the first batch.  wcnt: the longest part of the warp's rows (a bound
+// of the loop that every lane shares; a slot past it would only occupy the
+// float64 pipe with predicated-off operations).
+template <int LPR, bool UPPER, int MODE, typename T>
+__device__ __forceinline__ T part_sum(T acc, PartBatch<LPR, T>& B, int64_t base, int cnt, int wcnt,
+                                      int last, int lane, const int32_t* __restrict__ scol,
+                                      const T* __restrict__ sval, const T* x, const T* b,
+                                      const T* __restrict__ dinv, int nrows, int32_t* err) {
+    constexpr int U = PartBatch<LPR, T>::U;
+    for (int it = 0; it * U * LPR < wcnt; ++it) {
+        if (it > 0) B.template load<UPPER>(it, base, cnt, last, lane, scol, sval, nrows, err);
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v[u] = T(0);
+            if ((it * U + u) * LPR < wcnt && B.j[u] >= 0) v[u] = nbr_value<MODE, T>(B.j[u], x, b, dinv);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if ((it * U + u) * LPR < wcnt && B.j[u] >= 0) acc = fmad(-B.a[u], v[u], acc);
+    }
+    return acc;
+}
+
+// Both sums of a group of G lanes in log2(G) + 1 exchanges: even lanes carry
+// the first sum, odd lanes the second; every lane returns with both.
+template <int G, typename T>
+__device__ __forceinline__ void group_sum2(T& p, T& q) {
+    if (G == 1) return;
+    const bool odd = threadIdx.x & 1;
+    T keep = odd ? q : p;
+    keep += __shfl_xor_sync(0xffffffffu, odd ? p : q, 1);
+#pragma unroll
+    for (int off = 2; off < G; off <<= 1) keep += __shfl_xor_sync(0xffffffffu, keep, off);
+    const T other = __shfl_xor_sync(0xffffffffu, keep, 1);
+    p = odd ? other : keep;
+    q = odd ? keep : other;
+}
+
+// The update of one row by its LPR lanes: s and x = (s - U x) / A_ii as far as
+// PART asks for them.  acc(): b_i (kPartLower, kPartBoth) or s_i (kPartUpper),
+// read after wait().
+template <int LPR, int PART, int MODE, typename T, typename AccF, typename Wait>
+__device__ __forceinline__ void split_row(int64_t base, int low, int up, int last, int lane,
+                                          const int32_t* __restrict__ scol,
+                                          const T* __restrict__ sval, const T* x, const T* b,
+                                          const T* __restrict__ dinv, int nrows, int32_t* err,
+                                          AccF acc, Wait wait, T& s, T& sx) {
+    constexpr bool kLow = PART != kPartUpper, kUp = PART != kPartLower;
+    const int wlow = kLow ? (int)__reduce_max_sync(0xffffffffu, (unsigned)low) : 0;
+    const int wup = kUp ? (int)__reduce_max_sync(0xffffffffu, (unsigned)up) : 0;
+    PartBatch<LPR, T> BL, BU;
+    if (kLow) BL.template load<false>(0, base, low, last, lane, scol, sval, nrows, err);
+    if (kUp) BU.template load<true>(0, base, up, last, lane, scol, sval, nrows, err);
+    wait();
+    const T a0 = lane == 0 ? acc() : T(0);
+    s = kLow ? part_sum<LPR, false, MODE, T>(a0, BL, base, low, wlow, last, lane, scol, sval, x, b,
+                                             dinv, nrows, err)
+             : T(0);
+    sx = kUp ? part_sum<LPR, true, MODE, T>(kLow ? T(0) : a0, BU, base, up, wup, last, lane, scol,
+                                            sval, x, b, dinv, nrows, err)
+             : T(0);
+    if (PART == kPartBoth) {
+        group_sum2<LPR>(s, sx);
+        sx = s + sx;
+    } else if (kLow) {
+        s = group_sum<LPR>(s);
+        sx = s;
+    } else {
+        sx = group_sum<LPR>(sx);
+    }
+}
+
+// First two forward passes from a zero guess: colour 0 is x = b / A_ii, colour
+// 1 reads its lower part with the colour-0 values b_j / A_jj recomputed, and
+// keeps s.  Arguments: c1 = jmax, c2 = r1, dv = 1/A_ii, out = s.
+template <int LPR, typename T>
+struct SplitFirstBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int c1 = a.jmax, c2 = a.r1;
+        const T* __restrict__ dinv = static_cast<const T*>(a.dv);
+        const T* b = static_cast<const T*>(a.b);
+        T* x = static_cast<T*>(a.x);
+        T* sv = static_cast<T*>(a.out);
+        pdl_launch_dependents();
+        const RowOf<LPR> R(0, c2, bid);
+        const int rr = R.valid ? R.row : 0;
+        const int low = (R.valid && rr >= c1) ? (int)a.rlow[rr] : 0;
+        const int64_t base = (int64_t)(rr >> 5) * a.sw + (rr & 31);
+        const T di = R.valid ? dinv[rr] : T(0);
+        T s, sx;
+        split_row<LPR, kPartLower, kNbrFirst, T>(base, low, 0, 0, R.lane, a.scol,
+                                                 static_cast<const T*>(a.sval), x, b, dinv, a.n, a.err,
+                                                 [&] { return R.valid ? b[rr] : T(0); }, PdlWait(), s, sx);
+        if (R.valid && R.lane == 0) {
+            x[rr] = s * di;
+            if (rr >= c1) sv[rr] = s;
+        }
+    }
+};
+
+// One colour pass over the rows [r0, r1).  Arguments: r0, r1, width, dv =
+// 1/A_ii, b = b (kPartLower, kPartBoth) or s (kPartUpper; b for colour 0, whose
+// lower parts are empty), out = s, written where set.
+template <int LPR, typename T, int PART>
+struct SplitPassBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int r0 = a.r0, r1 = a.r1;
+        const T* __restrict__ dinv = static_cast<const T*>(a.dv);
+        const T* b = static_cast<const T*>(a.b);
+        T* x = static_cast<T*>(a.x);
+        T* sv = static_cast<T*>(a.out);
+        pdl_launch_dependents();
+        const RowOf<LPR> R(r0, r1, bid);
+        const int rr = R.valid ? R.row : r0;
+        const int low = R.valid ? (int)a.rlow[rr] : 0;
+        const int up = (R.valid && PART != kPartLower) ? (int)a.rlen[rr] - low : 0;
+        const int64_t base = (int64_t)(rr >> 5) * a.sw + (rr & 31);
+        const T di = R.valid ? dinv[rr] : T(0);
+        T s, sx;
+        split_row<LPR, PART, kNbrX, T>(base, low, up, a.width - 1, R.lane, a.scol,
+                                       static_cast<const T*>(a.sval), x, nullptr, nullptr, a.n, a.err,
+                                       [&] { return R.valid ? b[rr] : T(0); }, PdlWait(), s, sx);
+        if (R.valid && R.lane == 0) {
+            x[rr] = sx * di;
+            if (PART != kPartUpper && sv) sv[rr] = s;
+        }
+    }
+};
+
+// r = b - A x = (b - s) - L x for the rows [r0, n) after the backward sweep,
+// written over s.  Arguments: r0, r1 = n, out = s and r.
+template <int LPR, typename T>
+struct SplitResidualBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int r0 = a.r0, n = a.r1;
+        const T* b = static_cast<const T*>(a.b);
+        const T* x = static_cast<const T*>(a.x);
+        T* r = static_cast<T*>(a.out);
+        pdl_launch_dependents();
+        const RowOf<LPR> R(r0, n, bid);
+        const int rr = R.valid ? R.row : r0;
+        const int low = R.valid ? (int)a.rlow[rr] : 0;
+        const int64_t base = (int64_t)(rr >> 5) * a.sw + (rr & 31);
+        T s, sx;
+        split_row<LPR, kPartLower, kNbrX, T>(base, low, 0, 0, R.lane, a.scol,
+                                             static_cast<const T*>(a.sval), x, nullptr, nullptr, a.n,
+                                             a.err, [&] { return R.valid ? b[rr] - r[rr] : T(0); },
+                                             PdlWait(), s, sx);
+        if (R.valid && R.lane == 0) r[rr] = s;
+    }
+};
+
+// ---------------------------------------------------------------------------
 // Dependency-driven sweep (see SweepPlan in device.h): every colour pass of a
 // symmetric Gauss-Seidel sweep in one launch, one block per item of rows.
 // The rows of an item are updated exactly as PassBody (and, for the first
@@ -436,17 +629,20 @@ __device__ __forceinline__ void red_release_add_u64(unsigned long long* p, unsig
 // increasing order, so the block holding the smallest unfinished item always
 // has what it waits for: the sweep cannot deadlock.  The launch's epoch comes
 // from a counter of block arrivals (G per launch).
-template <int LPR, typename T>
+// SPLIT: the level's rows are split (sv = s); the passes then read the parts
+// that SplitPassBody reads.
+template <int LPR, typename T, bool SPLIT>
 __global__ void __launch_bounds__(kBlock) k_sweep(int npass, const SweepPass* __restrict__ passes,
                                                   int items, const int32_t* __restrict__ dep_ptr,
                                                   const int32_t* __restrict__ dep, uint32_t* flag,
                                                   unsigned long long* done,
                                                   unsigned long long* arrive, int32_t* failed,
                                                   int64_t sw, const uint16_t* __restrict__ rlen,
+                                                  const uint16_t* __restrict__ rlow,
                                                   const int32_t* __restrict__ scol,
                                                   const T* __restrict__ sval,
                                                   const T* __restrict__ dinv, const T* b, T* x,
-                                                  int32_t* err, int nrows) {
+                                                  T* sv, int32_t* err, int nrows) {
     __shared__ SweepPass sp[kSweepMaxPasses];
     __shared__ uint32_t s_epoch;
     __shared__ int s_ok;
@@ -508,11 +704,38 @@ __global__ void __launch_bounds__(kBlock) k_sweep(int npass, const SweepPass* __
             }
             __syncthreads();
         };
-        const T v = row_update<LPR, kNbrX, T>(base, len, (int)(sw >> 5), lane, P.jmax, scol, sval, x,
-                                              b, dinv, nrows, err,
-                                              [&] { return valid ? b[rr] : T(0); }, wait);
-        if (!s_ok) return;
-        if (valid && lane == 0) x[rr] = v * di;
+        T v, s = T(0);
+        if (SPLIT) {
+            const int low = (valid && !P.first) ? (int)rlow[rr] : 0, last = (int)(sw >> 5) - 1;
+            const int part = P.part;
+            // (s is written for every forward pass: a row's s is read by the
+            // block that updates the same rows in the backward pass)
+            if (part == kPartUpper) {
+                const T* src = P.r0 == 0 ? b : sv;
+                split_row<LPR, kPartUpper, kNbrX, T>(base, low, len - low, last, lane, scol, sval, x,
+                                                     nullptr, nullptr, nrows, err,
+                                                     [&] { return valid ? src[rr] : T(0); }, wait, s, v);
+            } else if (part == kPartBoth) {
+                split_row<LPR, kPartBoth, kNbrX, T>(base, low, len - low, last, lane, scol, sval, x,
+                                                    nullptr, nullptr, nrows, err,
+                                                    [&] { return valid ? b[rr] : T(0); }, wait, s, v);
+            } else {
+                split_row<LPR, kPartLower, kNbrX, T>(base, low, 0, last, lane, scol, sval, x, nullptr,
+                                                     nullptr, nrows, err,
+                                                     [&] { return valid ? b[rr] : T(0); }, wait, s, v);
+            }
+            if (!s_ok) return;
+            if (valid && lane == 0) {
+                x[rr] = v * di;
+                if (part != kPartUpper) sv[rr] = s;
+            }
+        } else {
+            v = row_update<LPR, kNbrX, T>(base, len, (int)(sw >> 5), lane, P.jmax, scol, sval, x,
+                                          b, dinv, nrows, err,
+                                          [&] { return valid ? b[rr] : T(0); }, wait);
+            if (!s_ok) return;
+            if (valid && lane == 0) x[rr] = v * di;
+        }
         __syncthreads();
         if (threadIdx.x == 0) {   // release: the block's writes (ordered by the barrier) first
             st_release_u32(flag + item, epoch);
@@ -622,10 +845,12 @@ __device__ __forceinline__ int64_t ld_offset(const int64_t* p) {
 template <typename T>
 __device__ bool stage_own_width(int64_t slice0, int nsl, const int64_t* soff, const int32_t* ccol,
                                 const T* cval, int32_t* s_col, T* s_val, uint64_t* bar, int32_t* err,
-                                int& loc) {
+                                int& loc, int& last) {
     const int w = (int)(threadIdx.x >> 5);
     const int64_t e0 = ld_offset(soff + slice0);
-    loc = (int)(ld_offset(soff + slice0 + min(w, nsl)) - e0) + (int)(threadIdx.x & 31);
+    const int64_t ew = ld_offset(soff + slice0 + min(w, nsl));
+    loc = (int)(ew - e0) + (int)(threadIdx.x & 31);
+    last = (int)((ld_offset(soff + slice0 + min(w + 1, nsl)) - ew) >> 5) - 1;
     if (threadIdx.x == 0) {
         const uint32_t ub = smem_u32(bar);
         const uint32_t ent = (uint32_t)(ld_offset(soff + slice0 + nsl) - e0);
@@ -679,8 +904,8 @@ struct FineTile {
     int64_t slice0;
     int nsl;
     int row;
-    int loc;          // offset of this row's entry 0 in the tiles (entry k at loc + 32 k),
-                      // set by the staging (stage_tile)
+    int loc;          // offset of this row's slot 0 in the tiles (slot k at loc + 32 k), and
+    int last;         // its last slot, set by the staging (stage_tile)
     int32_t* s_col;
     T* s_val;
     __device__ FineTile(int r0, int64_t nslices, int64_t cap, unsigned char* smem, int bid) {
@@ -688,6 +913,7 @@ struct FineTile {
         nsl = (int)min((int64_t)kSlicesPerBlock, nslices - slice0);
         row = (int)(slice0 * 32) + (int)threadIdx.x;
         loc = (int)(threadIdx.x & 31);
+        last = 0;
         s_col = reinterpret_cast<int32_t*>(smem);
         s_val = reinterpret_cast<T*>(smem + (size_t)cap * sizeof(int32_t));
     }
@@ -708,6 +934,19 @@ __device__ __forceinline__ T fine_row(const FineTile<T>& F, int len, int jmax, N
     return acc;
 }
 
+// acc - sum over the staged lower (upper) part of this thread's row
+template <bool UPPER, typename T>
+__device__ __forceinline__ T fine_part(const FineTile<T>& F, int cnt, const T* x, T acc, int nrows,
+                                       int32_t* err) {
+#pragma unroll 4
+    for (int t = 0; t < cnt; ++t) {
+        const int e = F.loc + 32 * (UPPER ? F.last - t : t);
+        const int j = F.s_col[e];
+        if (index_ok(j, nrows, err)) acc = fmad(-F.s_val[e], x[j], acc);
+    }
+    return acc;
+}
+
 // Stage the block's slices (per-slice widths when soff is set, else the
 // common width) and return whether the copies completed.
 template <typename T>
@@ -715,7 +954,8 @@ __device__ __forceinline__ bool stage_tile(FineTile<T>& F, const VArgs& a, uint6
     const T* sval = static_cast<const T*>(a.sval);
     if (a.soff)
         return stage_own_width(F.slice0, F.nsl, a.soff, a.scol, sval, F.s_col, F.s_val, bar, a.err,
-                               F.loc);
+                               F.loc, F.last);
+    F.last = a.width - 1;
     return stage_slices(F.slice0, F.nsl, a.width, a.scol, sval, F.s_col, F.s_val, bar, a.err, F.loc);
 }
 
@@ -810,6 +1050,58 @@ struct FineResidualBody {
         if (!valid) return;
         r[F.row] = fine_row<T>(F, len, n, [&](int j) { return x[j]; }, fmad(-dg, x[F.row], b[F.row]),
                                a.n, a.err);
+    }
+};
+
+// The staged colour pass and residual of a split level; arguments as
+// SplitPassBody and SplitResidualBody, with width, nslices, cap, soff as
+// FinePassBody.
+template <typename T, int PART>
+struct FineSplitPassBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int r0 = a.r0, r1 = a.r1;
+        const T* __restrict__ dinv = static_cast<const T*>(a.dv);
+        const T* b = static_cast<const T*>(a.b);
+        T* x = static_cast<T*>(a.x);
+        T* sv = static_cast<T*>(a.out);
+        extern __shared__ __align__(128) unsigned char smem[];
+        __shared__ uint64_t bar;
+        pdl_launch_dependents();
+        FineTile<T> F(r0, a.nslices, a.cap, smem, bid);
+        const bool valid = F.row >= r0 && F.row < r1;
+        const int low = valid ? (int)a.rlow[F.row] : 0;
+        const int up = (valid && PART != kPartLower) ? (int)a.rlen[F.row] - low : 0;
+        const T di = valid ? dinv[F.row] : T(0);
+        if (!stage_tile(F, a, &bar)) return;
+        pdl_wait();
+        if (!valid) return;
+        T s = b[F.row];
+        if (PART != kPartUpper) s = fine_part<false, T>(F, low, x, s, a.n, a.err);
+        const T sx = PART == kPartLower  ? s
+                     : PART == kPartBoth ? s + fine_part<true, T>(F, up, x, T(0), a.n, a.err)
+                                         : fine_part<true, T>(F, up, x, s, a.n, a.err);
+        x[F.row] = sx * di;
+        if (PART != kPartUpper && sv) sv[F.row] = s;
+    }
+};
+
+template <typename T>
+struct FineSplitResidualBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int r0 = a.r0, n = a.r1;
+        const T* b = static_cast<const T*>(a.b);
+        const T* x = static_cast<const T*>(a.x);
+        T* r = static_cast<T*>(a.out);
+        extern __shared__ __align__(128) unsigned char smem[];
+        __shared__ uint64_t bar;
+        pdl_launch_dependents();
+        FineTile<T> F(r0, a.nslices, a.cap, smem, bid);
+        const bool valid = F.row >= r0 && F.row < n;
+        const int low = valid ? (int)a.rlow[F.row] : 0;
+        if (!stage_tile(F, a, &bar)) return;
+        pdl_wait();
+        if (!valid) return;
+        r[F.row] = fine_part<false, T>(F, low, x, b[F.row] - r[F.row], a.n, a.err);
     }
 };
 
@@ -1562,6 +1854,15 @@ struct LevelArrays<float> {
         : sval(L.sval32), cval(L.cval32), dinv(L.dinv32), diag(L.diag32), t(L.t32) {}
 };
 
+// s = b - L x of a split level (the level's residual vector until the residual
+// takes its place)
+template <typename T>
+T* level_s(const DevLevel& L);
+template <>
+double* level_s<double>(const DevLevel& L) { return L.r; }
+template <>
+float* level_s<float>(const DevLevel& L) { return L.r32; }
+
 // dynamic shared memory a kernel gets without opting in, with room for its
 // static shared memory inside the 48 KB default
 constexpr size_t kDefaultDynSmem = 40 * 1024;
@@ -1630,6 +1931,7 @@ VArgs level_args(const DevLevel& L, const LevelArrays<T>& A) {
     a.nslices = fine_nslices(L);
     a.cap = L.stage_cap;
     a.rlen = L.rlen;
+    a.rlow = L.rlow;
     a.scol = L.scol;
     a.sval = A.sval;
     a.err = L.err;
@@ -1674,8 +1976,14 @@ void first_impl(const DevLevel& L, const T* b, T* x, T* bc_zero, int nc, cudaStr
             a.b = b;
             a.x = x;
             use_compact(L, A, a);
-            vlaunch<FinePassBody<T>>(fine_blocks(c1, c2), kFineBlock, fine_smem(L, sizeof(T)), s, a,
-                                     L.carve);
+            if (L.split) {
+                a.out = level_s<T>(L);
+                vlaunch<FineSplitPassBody<T, kPartLower>>(fine_blocks(c1, c2), kFineBlock,
+                                                          fine_smem(L, sizeof(T)), s, a, L.carve);
+            } else {
+                vlaunch<FinePassBody<T>>(fine_blocks(c1, c2), kFineBlock, fine_smem(L, sizeof(T)), s, a,
+                                         L.carve);
+            }
         }
         return;
     }
@@ -1686,15 +1994,35 @@ void first_impl(const DevLevel& L, const T* b, T* x, T* bc_zero, int nc, cudaStr
     a.dv = A.dinv;
     a.b = b;
     a.x = x;
+    if (L.split) {
+        a.out = level_s<T>(L);
+        AMG_LPR_DISPATCH(launch_lpr(L, c2),
+                         (vlaunch<SplitFirstBody<LPR, T>>(std::max(1, row_blocks(0, c2, LPR, L.block)),
+                                                          L.block, 0, s, a)));
+        return;
+    }
     AMG_LPR_DISPATCH(launch_lpr(L, c2),
                      (vlaunch<FirstBody<LPR, T>>(std::max(1, row_blocks(0, c2, LPR, L.block)), L.block,
                                                  0, s, a)));
 }
 
+template <typename T, int PART>
+void split_pass(const DevLevel& L, VArgs& a, const LevelArrays<T>& A, cudaStream_t s) {
+    if (L.lpr == kFine) {
+        use_compact(L, A, a);
+        vlaunch<FineSplitPassBody<T, PART>>(fine_blocks(a.r0, a.r1), kFineBlock, fine_smem(L, sizeof(T)),
+                                            s, a, L.carve);
+        return;
+    }
+    AMG_LPR_DISPATCH(launch_lpr(L, a.r1 - a.r0),
+                     (vlaunch<SplitPassBody<LPR, T, PART>>(row_blocks(a.r0, a.r1, LPR, L.block), L.block,
+                                                           0, s, a)));
+}
+
 // z_out / isq (fine level only): also write z = x * isq in float64 for the
 // rows of this pass (the float32 V-cycle's exit)
 template <typename T>
-void pass_impl(const DevLevel& L, int col, int jmax, const T* b, T* x, cudaStream_t s,
+void pass_impl(const DevLevel& L, int col, int jmax, RowPart part, const T* b, T* x, cudaStream_t s,
                double* z_out = nullptr, const double* isq = nullptr) {
     const LevelArrays<T> A(L);
     const int r0 = L.cptr[col], r1 = L.cptr[col + 1];
@@ -1706,6 +2034,18 @@ void pass_impl(const DevLevel& L, int col, int jmax, const T* b, T* x, cudaStrea
     a.dv = A.dinv;
     a.b = b;
     a.x = x;
+    if (L.split) {
+        // s of the forward pass: read by the backward pass over the colour
+        // (colour 0 has no lower part: s = b), and by the residual
+        if (part == kPartUpper) {
+            if (col > 0) a.b = level_s<T>(L);
+            return split_pass<T, kPartUpper>(L, a, A, s);
+        }
+        a.out = level_s<T>(L);
+        if (part == kPartLower) return split_pass<T, kPartLower>(L, a, A, s);
+        if (col == 0 || col == L.ncolours - 1) a.out = nullptr;
+        return split_pass<T, kPartBoth>(L, a, A, s);
+    }
     if (L.lpr == kFine) {
         a.z = z_out;
         a.isq = isq;
@@ -1742,7 +2082,18 @@ void residual_restrict_impl(const DevLevel& L, const T* b, const T* x, T* r, T* 
         }
         return;
     }
-    if (L.n > c1) {
+    if (L.n > c1 && L.split) {
+        a.out = r;
+        if (L.lpr == kFine) {
+            use_compact(L, A, a);
+            vlaunch<FineSplitResidualBody<T>>(fine_blocks(c1, L.n), kFineBlock, fine_smem(L, sizeof(T)),
+                                              s, a, L.carve);
+        } else {
+            AMG_LPR_DISPATCH(launch_lpr(L, L.n - c1),
+                             (vlaunch<SplitResidualBody<LPR, T>>(row_blocks(c1, L.n, LPR, L.block),
+                                                                 L.block, 0, s, a)));
+        }
+    } else if (L.n > c1) {
         a.out = r;
         if (L.lpr == kFine) {
             use_compact(L, A, a);
@@ -1785,7 +2136,7 @@ void prolong_impl(const DevLevel& L, const T* e, T* x, double omega, cudaStream_
     vlaunch<ProlongBody<T, SC>>(blocks_for(L.n - r0), kBlock, 0, s, a);
 }
 
-template <int LPR, typename T>
+template <int LPR, typename T, bool SPLIT>
 void sweep_launch(const DevLevel& L, const SweepPlan& P, const T* sval, const T* dinv, const T* b,
                   T* x, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
@@ -1798,10 +2149,11 @@ void sweep_launch(const DevLevel& L, const SweepPlan& P, const T* sval, const T*
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e =
-        cudaLaunchKernelEx(&cfg, k_sweep<LPR, T>, P.npass, (const SweepPass*)P.pass, P.items,
+        cudaLaunchKernelEx(&cfg, k_sweep<LPR, T, SPLIT>, P.npass, (const SweepPass*)P.pass, P.items,
                            (const int32_t*)P.dep_ptr, (const int32_t*)P.dep, P.flag, P.done,
                            P.arrive, P.failed, L.sw, (const uint16_t*)L.rlen,
-                           (const int32_t*)L.scol, sval, dinv, b, x, L.err, L.n);
+                           (const uint16_t*)L.rlow, (const int32_t*)L.scol, sval, dinv, b, x,
+                           level_s<T>(L), L.err, L.n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error{AMG_ECUDA, std::string("sweep launch (grid ") + std::to_string(P.grid) +
@@ -1815,15 +2167,21 @@ void sweep_impl(const DevLevel& L, const SweepPlan& P, const T* b, T* x, cudaStr
     if (P.items <= 0) return;
     if (L.lpr < 1 || P.rows * L.lpr != L.block || P.npass > kSweepMaxPasses || P.grid < 1)
         throw Error{AMG_EINVAL, "sweep plan does not match the level's launch shape"};
-    AMG_LPR_DISPATCH(L.lpr, (sweep_launch<LPR, T>(L, P, A.sval, A.dinv, b, x, s)));
+    if (L.split) {
+        AMG_LPR_DISPATCH(L.lpr, (sweep_launch<LPR, T, true>(L, P, A.sval, A.dinv, b, x, s)));
+    } else {
+        AMG_LPR_DISPATCH(L.lpr, (sweep_launch<LPR, T, false>(L, P, A.sval, A.dinv, b, x, s)));
+    }
 }
 
 template <int LPR>
 int sweep_blocks_per_sm(int block) {
-    int a = 0, b = 0;
-    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_sweep<LPR, double>, block, 0));
-    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sweep<LPR, float>, block, 0));
-    return std::min(a, b);
+    int a = 0, b = 0, c = 0, d = 0;
+    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_sweep<LPR, double, false>, block, 0));
+    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sweep<LPR, float, false>, block, 0));
+    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k_sweep<LPR, double, true>, block, 0));
+    AMG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d, k_sweep<LPR, float, true>, block, 0));
+    return std::min(std::min(a, b), std::min(c, d));
 }
 
 // co-resident blocks of the sweep kernel with `lanes` lanes per row and
@@ -1851,11 +2209,13 @@ void launch_first32(const DevLevel& L, const float* b, float* x, float* bc_zero,
                     cudaStream_t s) {
     first_impl<float>(L, b, x, bc_zero, nc, s);
 }
-void launch_pass(const DevLevel& L, int col, int jmax, const double* b, double* x, cudaStream_t s) {
-    pass_impl<double>(L, col, jmax, b, x, s);
+void launch_pass(const DevLevel& L, int col, int jmax, RowPart part, const double* b, double* x,
+                 cudaStream_t s) {
+    pass_impl<double>(L, col, jmax, part, b, x, s);
 }
-void launch_pass32(const DevLevel& L, int col, int jmax, const float* b, float* x, cudaStream_t s) {
-    pass_impl<float>(L, col, jmax, b, x, s);
+void launch_pass32(const DevLevel& L, int col, int jmax, RowPart part, const float* b, float* x,
+                   cudaStream_t s) {
+    pass_impl<float>(L, col, jmax, part, b, x, s);
 }
 void launch_first32_from64(const DevLevel& L, const double* r, const double* isq, float* b,
                            float* x, float* bc_zero, int nc, cudaStream_t s) {
@@ -1863,7 +2223,7 @@ void launch_first32_from64(const DevLevel& L, const double* r, const double* isq
 }
 void launch_pass32_to64(const DevLevel& L, int col, int jmax, const float* b, float* x,
                         double* z, const double* isq, cudaStream_t s) {
-    pass_impl<float>(L, col, jmax, b, x, s, z, isq);
+    pass_impl<float>(L, col, jmax, kPartBoth, b, x, s, z, isq);
 }
 void launch_residual_restrict(const DevLevel& L, const double* b, const double* x, double* r,
                               double* bc, cudaStream_t s) {

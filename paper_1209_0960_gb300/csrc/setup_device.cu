@@ -85,24 +85,35 @@ __global__ void k_galerkin(int nc, const int32_t* __restrict__ mptr, const int32
 
 // Copy row inv[r] of A into row r of the smoothing-order level: off-diagonal
 // entries (in their stored order, columns renumbered by perm) and diagonal.
+// With rlow set, the entries towards earlier colours (positions below r: equal
+// colours are not coupled) come first, in their stored order, and their number
+// goes to rlow.
 __global__ void k_reorder_rows(int n, const int32_t* __restrict__ inv, const int32_t* __restrict__ perm,
                                const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                const double* __restrict__ va, const int32_t* __restrict__ nrp,
                                int32_t* __restrict__ nci, double* __restrict__ nva,
-                               double* __restrict__ diag, double* __restrict__ dinv) {
+                               double* __restrict__ diag, double* __restrict__ dinv,
+                               uint16_t* __restrict__ rlow) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int i = inv[r];
-    int out = nrp[r];
+    int low = 0;
+    if (rlow) {
+        for (int k = rp[i]; k < rp[i + 1]; ++k) low += perm[ci[k]] < r ? 1 : 0;
+        rlow[r] = (uint16_t)low;
+    }
+    int out = nrp[r], up = nrp[r] + low;
     double d = 0.0;
     for (int k = rp[i]; k < rp[i + 1]; ++k) {
         const int j = ci[k];
         if (j == i) {
             d = va[k];
         } else {
-            nci[out] = perm[j];
-            nva[out] = va[k];
-            ++out;
+            const int pj = perm[j];
+            int& at = (rlow && pj > r) ? up : out;
+            nci[at] = pj;
+            nva[at] = va[k];
+            ++at;
         }
     }
     diag[r] = d;
@@ -110,19 +121,23 @@ __global__ void k_reorder_rows(int n, const int32_t* __restrict__ inv, const int
 }
 
 // Scatter the off-diagonal CSR rows into the SELL-32 arrays; padding entries
-// point at the row itself with value 0.
+// point at the row itself with value 0.  Split rows (rlow set) put their first
+// rlow entries into the slots 0, 1, ... and the others into width - 1,
+// width - 2, ...
 __global__ void k_csr_to_sell(int n, const int32_t* __restrict__ nrp, const int32_t* __restrict__ nci,
-                              const double* __restrict__ nva, int width,
-                              int32_t* __restrict__ scol, double* __restrict__ sval) {
+                              const double* __restrict__ nva, const uint16_t* __restrict__ rlow,
+                              int width, int32_t* __restrict__ scol, double* __restrict__ sval) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int64_t base = (int64_t)(r >> 5) * 32 * width + (r & 31);
     const int k0 = nrp[r], len = nrp[r + 1] - k0;
+    const int low = rlow ? (int)rlow[r] : len;
     for (int k = 0; k < width; ++k) {
         const int64_t e = base + 32 * (int64_t)k;
-        if (k < len) {
-            scol[e] = nci[k0 + k];
-            sval[e] = nva[k0 + k];
+        const int q = k < low ? k : low + (width - 1 - k);   // entry of the row in slot k
+        if (q < len) {
+            scol[e] = nci[k0 + q];
+            sval[e] = nva[k0 + q];
         } else {
             scol[e] = r;
             sval[e] = 0.0;
@@ -132,10 +147,12 @@ __global__ void k_csr_to_sell(int n, const int32_t* __restrict__ nrp, const int3
 
 // Copy the sliced arrays (common width W) into the layout with per-slice
 // widths: slice s starts at soff[s] and keeps K_s = (soff[s+1] - soff[s]) / 32
-// entries a row, entry k of lane i at soff[s] + 32 k + i (padding entries as
-// in the common layout: the row itself with value 0).  One thread per row.
+// entries a row, slot k of lane i at soff[s] + 32 k + i (padding entries as
+// in the common layout: the row itself with value 0); the upper parts of split
+// rows (rlow set) move to the end of their slice.  One thread per row.
 template <typename T>
-__global__ void k_sell_own_width(int n, int width, const int64_t* __restrict__ soff,
+__global__ void k_sell_own_width(int n, int width, const uint16_t* __restrict__ rlow,
+                                 const int64_t* __restrict__ soff,
                                  const int32_t* __restrict__ scol, const T* __restrict__ sval,
                                  int32_t* __restrict__ ccol, T* __restrict__ cval) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -143,9 +160,11 @@ __global__ void k_sell_own_width(int n, int width, const int64_t* __restrict__ s
     const int64_t src = (int64_t)(r >> 5) * 32 * width + (r & 31);
     const int64_t dst = soff[r >> 5] + (r & 31);
     const int ks = (int)((soff[(r >> 5) + 1] - soff[r >> 5]) >> 5);
+    const int low = rlow ? (int)rlow[r] : ks;
     for (int k = 0; k < ks; ++k) {
-        if (ccol) ccol[dst + 32 * (int64_t)k] = scol[src + 32 * (int64_t)k];
-        cval[dst + 32 * (int64_t)k] = sval[src + 32 * (int64_t)k];
+        const int64_t from = src + 32 * (int64_t)(k < low ? k : k + width - ks);
+        if (ccol) ccol[dst + 32 * (int64_t)k] = scol[from];
+        cval[dst + 32 * (int64_t)k] = sval[from];
     }
 }
 
@@ -500,7 +519,7 @@ void galerkin_device(const DevCsr& A, const HostCsr& Ah, const AggResult& R, Dev
 }
 
 void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<int32_t>& perm,
-                        DevArena& arena, DevLevel& L, cudaStream_t s) {
+                        bool split, DevArena& arena, DevLevel& L, cudaStream_t s) {
     const int32_t n = Ah.n;
     std::vector<int32_t> inv(n), nrp(n + 1, 0);
     std::vector<uint16_t> rlen(n);
@@ -542,6 +561,8 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
     const bool compact = width > 0 && 10 * L.padded > 11 * soff[nslices];
     L.stage_cap = compact ? 32 * window_max(kmax) : 256 * (int64_t)width;
     L.rlen = arena.alloc<uint16_t>(n);
+    L.split = split;
+    L.rlow = split ? arena.alloc<uint16_t>(n) : nullptr;
     L.scol = arena.alloc<int32_t>(L.padded);
     L.sval = arena.alloc<double>(L.padded);
     L.diag = arena.alloc<double>(n);
@@ -557,8 +578,8 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
     AMG_CUDA_TRY(cudaMemcpyAsync(d_nrp, nrp.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s));
     AMG_CUDA_TRY(cudaMemcpyAsync(L.rlen, rlen.data(), sizeof(uint16_t) * n, cudaMemcpyHostToDevice, s));
     k_reorder_rows<<<blocks_for(n), kBlock, 0, s>>>(n, d_inv, d_perm, A.rp, A.ci, A.va, d_nrp, d_nci,
-                                                    d_nva, L.diag, L.dinv);
-    k_csr_to_sell<<<blocks_for(n), kBlock, 0, s>>>(n, d_nrp, d_nci, d_nva, width, L.scol, L.sval);
+                                                    d_nva, L.diag, L.dinv, L.rlow);
+    k_csr_to_sell<<<blocks_for(n), kBlock, 0, s>>>(n, d_nrp, d_nci, d_nva, L.rlow, width, L.scol, L.sval);
     AMG_CUDA_TRY(cudaGetLastError());
     if (compact) {
         const int64_t ce = soff[nslices];
@@ -571,15 +592,26 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
         // rows past n in the last slice: padding entries of no row
         AMG_CUDA_TRY(cudaMemsetAsync(L.ccol, 0, sizeof(int32_t) * ce, s));
         AMG_CUDA_TRY(cudaMemsetAsync(L.cval, 0, sizeof(double) * ce, s));
-        k_sell_own_width<double><<<blocks_for(n), kBlock, 0, s>>>(n, width, L.soff, L.scol, L.sval,
-                                                                   L.ccol, L.cval);
+        k_sell_own_width<double><<<blocks_for(n), kBlock, 0, s>>>(n, width, L.rlow, L.soff, L.scol,
+                                                                  L.sval, L.ccol, L.cval);
         AMG_CUDA_TRY(cudaGetLastError());
     }
     // lanes per row: the staged one-row-per-thread kernels on sparse rows
     // (bandwidth bound), several lanes on the denser coarse rows (gather
-    // latency bound)
+    // latency bound).  Split levels read about half a row a pass, and the fewer
+    // rows a pass has, the more its time is one row's chain of loads, sums and
+    // instruction fetches.  Measured, V-cycle from the level, best shape against
+    // 4 lanes in blocks of 256: 6,619 rows 70.6 us (8 lanes, 128 threads) against
+    // 87.0; 8,204 rows 66.0 (8, 128) against 90.3; 51,913 rows 144.2 (4, 128)
+    // against 149.3; 77,212 rows 185.0 (2, 128) against 190.5; 610,622 rows
+    // 445.6 (1, 256) against 492.0; 1,671,533 rows 519.5 (1, 256) against 580.6.
     const double avg = n > 0 ? (double)L.nnz_off / n : 0.0;
-    L.lpr = (avg <= 7.0 && staged_fits(L)) ? 0 : avg <= 16.0 ? 4 : 8;
+    if (split) {
+        L.lpr = n <= 20000 ? 8 : n <= 60000 ? 4 : n <= 300000 ? 2 : 1;
+        L.block = n <= 300000 ? 128 : 256;
+    } else {
+        L.lpr = (avg <= 7.0 && staged_fits(L)) ? 0 : avg <= 16.0 ? 4 : 8;
+    }
     L.lpr_wide = L.lpr;
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
 }
@@ -663,7 +695,7 @@ void build_level_fp32(DevLevel& L, const double* coarse_diag, DevArena& arena, c
         const int64_t ce = L.stage_entries;
         L.cval32 = arena.alloc<float>(ce);
         AMG_CUDA_TRY(cudaMemsetAsync(L.cval32, 0, sizeof(float) * ce, s));
-        k_sell_own_width<float><<<blocks_for(n), kBlock, 0, s>>>(n, L.width, L.soff, nullptr,
+        k_sell_own_width<float><<<blocks_for(n), kBlock, 0, s>>>(n, L.width, L.rlow, L.soff, nullptr,
                                                                   L.sval32, nullptr, L.cval32);
         AMG_CUDA_TRY(cudaGetLastError());
     }

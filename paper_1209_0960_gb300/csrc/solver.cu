@@ -108,32 +108,47 @@ std::vector<int32_t> smoothing_order(const HostLevel& h) {
 
 // colour pass over the m rows of colour col (z entries) reading neighbour
 // values at positions < jmax: entries, lengths, b, 1/A_ii, x written, and the
-// neighbour values once
-double pass_bytes(const DevLevel& L, int col, int jmax, int vb) {
+// neighbour values once.  On a split level only the entries of the part it
+// reads, both lengths, and s written by the forward passes.
+double pass_bytes(const DevLevel& L, int col, int jmax, int vb, RowPart part = kPartBoth) {
     const double m = L.cptr[col + 1] - L.cptr[col];
+    if (L.split) {
+        const double low = (double)L.clow[col], up = (double)L.cnnz[col] - low;
+        const double zl = part == kPartUpper ? 0.0 : low, zu = part == kPartLower ? 0.0 : up;
+        const double nb = std::min(zl, (double)L.cptr[col]) + std::min(zu, (double)L.n - L.cptr[col + 1]);
+        const bool writes_s = part != kPartUpper && col > 0 && (part == kPartLower || col < L.ncolours - 1);
+        return (zl + zu) * (vb + 4) + m * (4 + (writes_s ? 4.0 : 3.0) * vb) + nb * vb;
+    }
     const double z = (double)L.cnnz[col];
     const double nb = std::min(z, (double)jmax - (jmax > L.cptr[col] ? m : 0.0));
     return z * (vb + 4) + m * (2 + 3.0 * vb) + std::max(0.0, nb) * vb;
 }
 // fused first two forward passes: colour 0 reads b and 1/A_ii and writes x;
-// colour 1 reads its entries, b, 1/A_ii, writes x (colour-0 b and 1/A_ii are
-// already counted); the next level's right-hand side is zeroed when the
-// restriction is fused
+// colour 1 reads its entries, b, 1/A_ii, writes x and, on a split level, s
+// (colour-0 b and 1/A_ii are already counted); the next level's right-hand
+// side is zeroed when the restriction is fused
 double first_bytes(const DevLevel& L, int vb) {
     const double c1 = L.cptr[1];
     const double m1 = L.ncolours > 1 ? L.cptr[2] - L.cptr[1] : 0.0;
-    const double z1 = L.ncolours > 1 ? (double)L.cnnz[1] : 0.0;
-    return c1 * 3.0 * vb + z1 * (vb + 4) + m1 * (2 + 3.0 * vb) +
+    const double z1 = L.ncolours > 1 ? (double)(L.split ? L.clow[1] : L.cnnz[1]) : 0.0;
+    return c1 * 3.0 * vb + z1 * (vb + 4) + m1 * (2 + (L.split ? 4.0 : 3.0) * vb) +
            (L.fused_restrict ? (double)L.n_coarse * vb : 0.0);
 }
-// residual of the rows of colour >= 1 and restriction: entries, lengths, A_ii,
-// b, own x, colour-0 neighbour values once, then either the coarse index (and
-// weight) and one atomic add per aggregate (fused) or the written r, the
-// restriction lists, r again and the coarse right-hand side
+// residual of the rows of colour >= 1 and restriction: entries (the lower
+// parts of a split level), lengths, A_ii (s), b, own x, earlier colours' values
+// once, then either the coarse index (and weight) and one atomic add per
+// aggregate (fused) or the written r, the restriction lists, r again and the
+// coarse right-hand side
 double residual_restrict_bytes(const DevLevel& L, int vb, bool scaled) {
     const double m = L.n - L.cptr[1];
-    const double z = (double)(L.nnz_off - L.cnnz[0]);
-    const double core = z * (vb + 4) + m * (2 + 3.0 * vb) + std::min(z, (double)L.cptr[1]) * vb;
+    double z = (double)(L.nnz_off - L.cnnz[0]), nb = (double)L.cptr[1], own = 3.0;
+    if (L.split) {
+        z = 0.0;
+        for (int64_t low : L.clow) z += (double)low;
+        nb = (double)L.cptr[L.ncolours - 1];
+        own = 2.0;
+    }
+    const double core = z * (vb + 4) + m * (2 + own * vb) + std::min(z, nb) * vb;
     if (L.fused_restrict) return core + m * (4 + (scaled ? 4 : 0)) + (double)L.n_coarse * 2 * vb;
     return core + m * vb + m * (4 + vb + (scaled ? 4 : 0)) + 4.0 * (L.n_coarse + 1) +
            (double)L.n_coarse * vb;
@@ -152,12 +167,12 @@ double level_vcycle_bytes(const DevLevel& L, bool coarsest, int vb, int mb = 8) 
     const bool scaled = vb == 4;
     const int C = L.ncolours;
     double t = first_bytes(L, vb);
-    for (int col = 2; col < C; ++col) t += pass_bytes(L, col, L.cptr[col], vb);
-    for (int col = C - 2; col >= 0; --col) t += pass_bytes(L, col, L.n, vb);
+    for (int col = 2; col < C; ++col) t += pass_bytes(L, col, L.cptr[col], vb, kPartLower);
+    for (int col = C - 2; col >= 0; --col) t += pass_bytes(L, col, L.n, vb, kPartUpper);
     t += residual_restrict_bytes(L, vb, scaled);
     t += prolong_bytes(L, vb, scaled);
     for (int col = 0; col < C; ++col) t += pass_bytes(L, col, L.n, vb);
-    for (int col = C - 2; col >= 0; --col) t += pass_bytes(L, col, L.n, vb);
+    for (int col = C - 2; col >= 0; --col) t += pass_bytes(L, col, L.n, vb, kPartUpper);
     return t;
 }
 
@@ -283,8 +298,8 @@ struct Prec<float> {
 
 inline void k_first(const DevLevel& L, const double* b, double* x, double* bc, int nc, cudaStream_t s) { launch_first(L, b, x, bc, nc, s); }
 inline void k_first(const DevLevel& L, const float* b, float* x, float* bc, int nc, cudaStream_t s) { launch_first32(L, b, x, bc, nc, s); }
-inline void k_pass(const DevLevel& L, int col, int jmax, const double* b, double* x, cudaStream_t s) { launch_pass(L, col, jmax, b, x, s); }
-inline void k_pass(const DevLevel& L, int col, int jmax, const float* b, float* x, cudaStream_t s) { launch_pass32(L, col, jmax, b, x, s); }
+inline void k_pass(const DevLevel& L, int col, int jmax, RowPart part, const double* b, double* x, cudaStream_t s) { launch_pass(L, col, jmax, part, b, x, s); }
+inline void k_pass(const DevLevel& L, int col, int jmax, RowPart part, const float* b, float* x, cudaStream_t s) { launch_pass32(L, col, jmax, part, b, x, s); }
 inline void k_resres(const DevLevel& L, const double* b, const double* x, double* r, double* bc, cudaStream_t s) { launch_residual_restrict(L, b, x, r, bc, s); }
 inline void k_resres(const DevLevel& L, const float* b, const float* x, float* r, float* bc, cudaStream_t s) { launch_residual_restrict32(L, b, x, r, bc, s); }
 inline void k_prolong(const DevLevel& L, const double* e, double* x, double w, cudaStream_t s) { launch_prolong(L, e, x, w, s); }
@@ -325,8 +340,8 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
     if (L.sweep) {
         // the whole pre-smoother as one dependency-driven kernel
         double bytes = first_bytes(L, vb);
-        for (int col = 2; col < C; ++col) bytes += pass_bytes(L, col, L.cptr[col], vb);
-        for (int col = C - 2; col >= 0; --col) bytes += pass_bytes(L, col, L.n, vb);
+        for (int col = 2; col < C; ++col) bytes += pass_bytes(L, col, L.cptr[col], vb, kPartLower);
+        for (int col = C - 2; col >= 0; --col) bytes += pass_bytes(L, col, L.n, vb, kPartUpper);
         ProfScope ps(c, kind, bytes);
         k_sweep(L, *L.plan_pre, b, x, s);
     } else {
@@ -336,14 +351,14 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
             k_first(L, b, x, L.fused_restrict ? P::b(N) : (T*)nullptr, N.n, s);
         }
         for (int col = 2; col < C; ++col) {
-            ProfScope ps(c, kind, pass_bytes(L, col, L.cptr[col], vb));
+            ProfScope ps(c, kind, pass_bytes(L, col, L.cptr[col], vb, kPartLower));
             vkey(0, l, 2 + col);
-            k_pass(L, col, L.cptr[col], b, x, s);
+            k_pass(L, col, L.cptr[col], kPartLower, b, x, s);
         }
         for (int col = C - 2; col >= 0; --col) {
-            ProfScope ps(c, kind, pass_bytes(L, col, L.n, vb));
+            ProfScope ps(c, kind, pass_bytes(L, col, L.n, vb, kPartUpper));
             vkey(0, l, 100 + (C - 2 - col));
-            k_pass(L, col, L.n, b, x, s);
+            k_pass(L, col, L.n, kPartUpper, b, x, s);
         }
     }
     {
@@ -361,7 +376,7 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
         // the whole post-smoother as one dependency-driven kernel
         double bytes = 0.0;
         for (int col = 0; col < C; ++col) bytes += pass_bytes(L, col, L.n, vb);
-        for (int col = C - 2; col >= 0; --col) bytes += pass_bytes(L, col, L.n, vb);
+        for (int col = C - 2; col >= 0; --col) bytes += pass_bytes(L, col, L.n, vb, kPartUpper);
         ProfScope ps(c, kind, bytes);
         k_sweep(L, *L.plan_post, b, x, s);
         return;
@@ -369,12 +384,12 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
     for (int col = 0; col < C; ++col) {
         ProfScope ps(c, kind, pass_bytes(L, col, L.n, vb));
         vkey(1, 64 - l, 2 + col);
-        k_pass(L, col, L.n, b, x, s);
+        k_pass(L, col, L.n, kPartBoth, b, x, s);
     }
     for (int col = C - 2; col >= 0; --col) {
-        ProfScope ps(c, kind, pass_bytes(L, col, L.n, vb));
+        ProfScope ps(c, kind, pass_bytes(L, col, L.n, vb, kPartUpper));
         vkey(1, 64 - l, 100 + (C - 2 - col));
-        k_pass(L, col, L.n, b, x, s);
+        k_pass(L, col, L.n, kPartUpper, b, x, s);
     }
 }
 
@@ -401,12 +416,12 @@ void vcycle32_fused(amg_ctx* c, const double* r, double* z) {
     for (int col = 2; col < C; ++col) {
         ProfScope ps(c, kKGsL0, pass_bytes(L, col, L.cptr[col], 4));
         vkey(0, 0, 2 + col);
-        launch_pass32(L, col, L.cptr[col], b, x, s);
+        launch_pass32(L, col, L.cptr[col], kPartBoth, b, x, s);
     }
     for (int col = C - 2; col >= 0; --col) {
         ProfScope ps(c, kKGsL0, pass_bytes(L, col, L.n, 4));
         vkey(0, 0, 100 + (C - 2 - col));
-        launch_pass32(L, col, L.n, b, x, s);
+        launch_pass32(L, col, L.n, kPartBoth, b, x, s);
     }
     {
         ProfScope ps(c, kKResidualL0, residual_restrict_bytes(L, 4, true));
@@ -425,7 +440,7 @@ void vcycle32_fused(amg_ctx* c, const double* r, double* z) {
         ProfScope ps(c, kKGsL0, pass_bytes(L, col, L.n, 4) + (last ? 16.0 * (L.cptr[col + 1] - L.cptr[col]) : 0.0));
         vkey(1, 64, 2 + col);
         if (last) launch_pass32_to64(L, col, L.n, b, x, z, isq, s);
-        else launch_pass32(L, col, L.n, b, x, s);
+        else launch_pass32(L, col, L.n, kPartBoth, b, x, s);
     }
     for (int col = C - 2; col >= 0; --col) {
         ProfScope ps(c, kKGsL0, pass_bytes(L, col, L.n, 4) + 16.0 * (L.cptr[col + 1] - L.cptr[col]));
@@ -608,23 +623,24 @@ void plan_sweep(amg_ctx* c, int l, int rows, bool pre, SweepPlan& P) {
     // the passes, and the colour of each
     std::vector<SweepPass> pass;
     std::vector<int> pcol;
-    auto add = [&](int col, int32_t jmax, int first) {
+    auto add = [&](int col, int32_t jmax, int first, RowPart part) {
         if (tiles[col] == 0) return;
         SweepPass q;
         q.r0 = L.cptr[col];
         q.r1 = L.cptr[col + 1];
         q.jmax = jmax;
         q.first = first;
+        q.part = part;
         q.tiles = tiles[col];
         q.item0 = pass.empty() ? 0 : pass.back().item0 + pass.back().tiles;
         pass.push_back(q);
         pcol.push_back(col);
     };
     for (int col = 0; col < C; ++col) {
-        if (pre) add(col, col == 0 ? 0 : L.cptr[col], col == 0 ? 1 : 0);
-        else add(col, n, 0);
+        if (pre) add(col, col == 0 ? 0 : L.cptr[col], col == 0 ? 1 : 0, kPartLower);
+        else add(col, n, 0, kPartBoth);
     }
-    for (int col = C - 2; col >= 0; --col) add(col, n, 0);
+    for (int col = C - 2; col >= 0; --col) add(col, n, 0, kPartUpper);
     const int np = (int)pass.size();
     if (np > kSweepMaxPasses) throw Error{AMG_EINVAL, "too many colour passes for a sweep kernel"};
     const int32_t items = np ? pass.back().item0 + pass.back().tiles : 0;
@@ -1613,7 +1629,7 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     for (int l = 0; l < nlev; ++l) {
         HostLevel& h = c->hl[l];
         DevLevel& L = c->dl[l];
-        build_level_device(dA[l], h.A, h.perm, c->mem, L, s);
+        build_level_device(dA[l], h.A, h.perm, l > 0 && l < nlev - 1 && h.ncolours >= 3, c->mem, L, s);
         L.x = c->mem.alloc<double>(L.n);
         L.b = c->mem.alloc<double>(L.n);
         L.r = c->mem.alloc<double>(L.n);
@@ -1630,6 +1646,15 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
             L.cnnz[h.colour[i]] += h.A.rp[i + 1] - h.A.rp[i] - 1;
         }
         for (int col = 0; col < h.ncolours; ++col) L.cptr[col + 1] += L.cptr[col];
+        if (L.split) {
+            std::vector<uint16_t> low(L.n);
+            AMG_CUDA_TRY(cudaMemcpyAsync(low.data(), L.rlow, sizeof(uint16_t) * L.n,
+                                         cudaMemcpyDeviceToHost, s));
+            AMG_CUDA_TRY(cudaStreamSynchronize(s));
+            L.clow.assign(h.ncolours, 0);
+            for (int col = 0; col < h.ncolours; ++col)
+                for (int32_t r = L.cptr[col]; r < L.cptr[col + 1]; ++r) L.clow[col] += low[r];
+        }
         const std::vector<int32_t>& pn = c->hl[l + 1].perm;
         const int32_t nc = h.agg.nc;
         L.n_coarse = nc;
@@ -2124,14 +2149,17 @@ int amg_debug_set_column(amg_ctx* c, int32_t l, int32_t row, int32_t k, int32_t 
         AMG_CUDA_TRY(cudaMemcpy(&rl, L.rlen + r, sizeof(uint16_t), cudaMemcpyDeviceToHost));
         const int32_t len = rl;
         if (k < 0 || k >= len) throw Error{AMG_EINVAL, "k out of range of the row's entries"};
-        const int64_t e = (int64_t)(r >> 5) * L.sw + 32 * (int64_t)k + (r & 31);
+        uint16_t low = rl;   // slot of entry k: from the end for the upper part of a split row
+        if (L.split) AMG_CUDA_TRY(cudaMemcpy(&low, L.rlow + r, sizeof(uint16_t), cudaMemcpyDeviceToHost));
+        const auto slot = [&](int64_t width) { return k < (int)low ? (int64_t)k : width - 1 - (k - (int)low); };
+        const int64_t e = (int64_t)(r >> 5) * L.sw + 32 * slot(L.width) + (r & 31);
         AMG_CUDA_TRY(cudaStreamSynchronize(c->stream));
         AMG_CUDA_TRY(cudaMemcpy(L.scol + e, &col, sizeof(int32_t), cudaMemcpyHostToDevice));
         if (L.soff) {
             // the same entry in the copy with per-slice widths
-            int64_t pos = 0;
-            AMG_CUDA_TRY(cudaMemcpy(&pos, L.soff + (r >> 5), sizeof(int64_t), cudaMemcpyDeviceToHost));
-            pos += 32 * (int64_t)k + (r & 31);
+            int64_t so[2] = {};
+            AMG_CUDA_TRY(cudaMemcpy(so, L.soff + (r >> 5), 2 * sizeof(int64_t), cudaMemcpyDeviceToHost));
+            const int64_t pos = so[0] + 32 * slot((so[1] - so[0]) / 32) + (r & 31);
             AMG_CUDA_TRY(cudaMemcpy(L.ccol + pos, &col, sizeof(int32_t), cudaMemcpyHostToDevice));
         }
         drop_graphs(c);
