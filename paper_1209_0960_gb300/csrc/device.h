@@ -364,8 +364,9 @@ struct CgWork {
 // scalars; it also counts its own evaluations and stops at maxit.
 void launch_cg_continue(cudaGraphConditionalHandle h, PcgScalars* sc, cudaStream_t s);
 extern thread_local bool t_launch_overlap;
-// grids above this many blocks launch without the overlap: a wide grid that
-// starts early only occupies the SMs its predecessor is still using
+// grids above this many blocks: CG kernels launch without the overlap (a wide
+// grid that starts early only occupies the SMs its predecessor is still
+// using), V-cycle kernels trigger their successor late
 extern int g_overlap_max_blocks;
 
 // Dynamic shared memory above the default needs a per-function attribute,
@@ -380,10 +381,12 @@ void raise_dyn_smem(void (*kernel)(KArgs...), size_t bytes) {
 
 // carve >= 0: the launch's preferred shared-memory carveout, in percent of
 // the SM's maximum shared memory (the rest of the unified L1/shared array is
-// L1 cache); -1: the driver's choice
+// L1 cache); -1: the driver's choice.  any_grid: the launch may overlap its
+// predecessor whatever its grid (V-cycle launches, whose wide grids trigger
+// late; see trigger_early in kernels.cu)
 template <typename... KArgs, typename... Args>
 void launch_kernel_carve(void (*kernel)(KArgs...), int grid, int block, size_t smem, int carve,
-                         cudaStream_t s, Args&&... args) {
+                         bool any_grid, cudaStream_t s, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
@@ -391,7 +394,7 @@ void launch_kernel_carve(void (*kernel)(KArgs...), int grid, int block, size_t s
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     unsigned n = 0;
-    if (t_launch_overlap && grid <= g_overlap_max_blocks) {
+    if (t_launch_overlap && (any_grid || grid <= g_overlap_max_blocks)) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n].val.programmaticStreamSerializationAllowed = 1;
         ++n;
@@ -415,7 +418,7 @@ void launch_kernel_carve(void (*kernel)(KArgs...), int grid, int block, size_t s
 template <typename... KArgs, typename... Args>
 void launch_kernel(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
                    Args&&... args) {
-    launch_kernel_carve(kernel, grid, block, smem, -1, s, std::forward<Args>(args)...);
+    launch_kernel_carve(kernel, grid, block, smem, -1, false, s, std::forward<Args>(args)...);
 }
 
 // Runs the staged kernels' bounded wait against an mbarrier that no copy
@@ -457,6 +460,8 @@ struct VArgs {
     double* z = nullptr;              // float64 output of the float32 V-cycle
     int32_t* err = nullptr;
     double omega = 0.0;
+    int32_t late = 0;                 // the launch lets its successor start after its wait
+                                      // (grids that do not fit on the SMs at once)
 };
 
 struct VRec;

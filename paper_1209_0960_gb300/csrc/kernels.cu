@@ -243,19 +243,37 @@ __host__ __device__ constexpr int lanes_of() { return LPR == kFine ? 1 : LPR; }
 template <int LPR>
 __host__ __device__ constexpr int unroll_of() { return LPR == 1 ? 24 : LPR == 2 ? 12 : kUnroll; }
 
+// When a V-cycle kernel lets its successor start.  A grid that fits on the
+// SMs at once triggers at entry: the successor's blocks are then resident and
+// have their matrix entries loaded when it ends.  In a wider grid (a.late) that
+// would put the successor's waiting blocks on SMs that its own last blocks
+// could use, so each block triggers after its wait: the successor starts as
+// the last wave drains, its launch and first loads under that wave's tail.
+// Late trigger against no overlap on wide grids, one iteration: layered
+// 192x160x145 float64 905 -> 837 us, anisotropic 256x224x209 mixed 1499 ->
+// 1457 us, log-normal 128^3 mixed 433 -> 421 us.
+__device__ __forceinline__ void trigger_early(const VArgs& a) {
+    if (!a.late) pdl_launch_dependents();
+}
+__device__ __forceinline__ void wait_and_trigger(const VArgs& a) {
+    pdl_wait();
+    if (a.late) pdl_launch_dependents();
+}
+
 struct PdlWait {
-    __device__ void operator()() const { pdl_wait(); }
+    const VArgs* a;
+    __device__ void operator()() const { wait_and_trigger(*a); }
 };
 
 // Wait: what the row does between loading its first batch of setup-time
 // entries and reading the first vector value (the predecessor's completion,
 // or a dependency wait).
-template <int LPR, int MODE, typename T, typename AccF, typename Wait = PdlWait>
+template <int LPR, int MODE, typename T, typename AccF, typename Wait>
 __device__ __forceinline__ T row_update(int64_t base, int len, int width, int lane, int jmax,
                                         const int32_t* __restrict__ scol,
                                         const T* __restrict__ sval, const T* x,
                                         const T* b, const T* __restrict__ dinv, int nrows,
-                                        int32_t* err, AccF acc, Wait wait = Wait()) {
+                                        int32_t* err, AccF acc, Wait wait) {
     static_assert(LPR != kFine, "the fine level uses the staged kernels");
     // every lane of the warp runs the same number of batches (the slice width
     // bounds every row length), so the warp-wide votes below see all 32 lanes
@@ -333,7 +351,7 @@ struct FirstBody {
         const T* __restrict__ dinv = static_cast<const T*>(a.dv);
         const T* b = static_cast<const T*>(a.b);
         T* x = static_cast<T*>(a.x);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(0, c2, bid);
         const int rr = R.valid ? R.row : 0;
         // colour-0 rows take no neighbour term (length 0: s = b_i exactly); every
@@ -343,7 +361,7 @@ struct FirstBody {
         const T di = R.valid ? dinv[rr] : T(0);
         const T s = row_update<LPR, kNbrFirst, T>(base, len, (int)(sw >> 5), R.lane, c1, scol, sval, x,
                                                    b, dinv, a.n, a.err,
-                                                   [&] { return R.valid ? b[rr] : T(0); });
+                                                   [&] { return R.valid ? b[rr] : T(0); }, PdlWait{&a});
         if (R.valid && R.lane == 0) x[rr] = s * di;
     }
 };
@@ -363,14 +381,14 @@ struct PassBody {
         const T* __restrict__ dinv = static_cast<const T*>(a.dv);
         const T* b = static_cast<const T*>(a.b);
         T* x = static_cast<T*>(a.x);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(r0, r1, bid);
         const int rr = R.valid ? R.row : r0;
         const int64_t base = (int64_t)(rr >> 5) * sw + (rr & 31);
         const T di = R.valid ? dinv[rr] : T(0);
         const T s = row_update<LPR, kNbrX, T>(base, R.valid ? (int)rlen[rr] : 0, (int)(sw >> 5),
                                               R.lane, jmax, scol, sval, x, b, dinv, a.n, a.err,
-                                              [&] { return R.valid ? b[rr] : T(0); });
+                                              [&] { return R.valid ? b[rr] : T(0); }, PdlWait{&a});
         if (R.valid && R.lane == 0) x[rr] = s * di;
     }
 };
@@ -388,7 +406,7 @@ struct ResidualBody {
         const T* b = static_cast<const T*>(a.b);
         const T* x = static_cast<const T*>(a.x);
         T* r = static_cast<T*>(a.out);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(r0, n, bid);
         const int rr = R.valid ? R.row : r0;
         const int64_t base = (int64_t)(rr >> 5) * sw + (rr & 31);
@@ -396,7 +414,7 @@ struct ResidualBody {
         const T v = row_update<LPR, kNbrX, T>(
             base, R.valid ? (int)rlen[rr] : 0, (int)(sw >> 5), R.lane, n, scol, sval, x,
             (const T*)nullptr, (const T*)nullptr, a.n, a.err,
-            [&] { return R.valid ? fmad(-dg, x[rr], b[rr]) : T(0); });
+            [&] { return R.valid ? fmad(-dg, x[rr], b[rr]) : T(0); }, PdlWait{&a});
         if (R.valid && R.lane == 0) r[rr] = v;
     }
 };
@@ -525,7 +543,7 @@ struct SplitFirstBody {
         const T* b = static_cast<const T*>(a.b);
         T* x = static_cast<T*>(a.x);
         T* sv = static_cast<T*>(a.out);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(0, c2, bid);
         const int rr = R.valid ? R.row : 0;
         const int low = (R.valid && rr >= c1) ? (int)a.rlow[rr] : 0;
@@ -534,7 +552,7 @@ struct SplitFirstBody {
         T s, sx;
         split_row<LPR, kPartLower, kNbrFirst, T>(base, low, 0, 0, R.lane, a.scol,
                                                  static_cast<const T*>(a.sval), x, b, dinv, a.n, a.err,
-                                                 [&] { return R.valid ? b[rr] : T(0); }, PdlWait(), s, sx);
+                                                 [&] { return R.valid ? b[rr] : T(0); }, PdlWait{&a}, s, sx);
         if (R.valid && R.lane == 0) {
             x[rr] = s * di;
             if (rr >= c1) sv[rr] = s;
@@ -553,7 +571,7 @@ struct SplitPassBody {
         const T* b = static_cast<const T*>(a.b);
         T* x = static_cast<T*>(a.x);
         T* sv = static_cast<T*>(a.out);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(r0, r1, bid);
         const int rr = R.valid ? R.row : r0;
         const int low = R.valid ? (int)a.rlow[rr] : 0;
@@ -563,7 +581,7 @@ struct SplitPassBody {
         T s, sx;
         split_row<LPR, PART, kNbrX, T>(base, low, up, a.width - 1, R.lane, a.scol,
                                        static_cast<const T*>(a.sval), x, nullptr, nullptr, a.n, a.err,
-                                       [&] { return R.valid ? b[rr] : T(0); }, PdlWait(), s, sx);
+                                       [&] { return R.valid ? b[rr] : T(0); }, PdlWait{&a}, s, sx);
         if (R.valid && R.lane == 0) {
             x[rr] = sx * di;
             if (PART != kPartUpper && sv) sv[rr] = s;
@@ -580,7 +598,7 @@ struct SplitResidualBody {
         const T* b = static_cast<const T*>(a.b);
         const T* x = static_cast<const T*>(a.x);
         T* r = static_cast<T*>(a.out);
-        pdl_launch_dependents();
+        trigger_early(a);
         const RowOf<LPR> R(r0, n, bid);
         const int rr = R.valid ? R.row : r0;
         const int low = R.valid ? (int)a.rlow[rr] : 0;
@@ -589,7 +607,7 @@ struct SplitResidualBody {
         split_row<LPR, kPartLower, kNbrX, T>(base, low, 0, 0, R.lane, a.scol,
                                              static_cast<const T*>(a.sval), x, nullptr, nullptr, a.n,
                                              a.err, [&] { return R.valid ? b[rr] - r[rr] : T(0); },
-                                             PdlWait(), s, sx);
+                                             PdlWait{&a}, s, sx);
         if (R.valid && R.lane == 0) r[rr] = s;
     }
 };
@@ -977,8 +995,8 @@ struct FineFirst0Body {
         T* bc_zero = static_cast<T*>(a.out);
         const double* r_in = a.rin;
         const double* __restrict__ isq = a.isq;
-        pdl_launch_dependents();
-        pdl_wait();
+        trigger_early(a);
+        wait_and_trigger(a);
         const int stride = gdim * blockDim.x;
         for (int i = bid * blockDim.x + threadIdx.x; i < nb; i += stride) {
             T bi;
@@ -1012,13 +1030,13 @@ struct FinePassBody {
         const double* __restrict__ isq = a.isq;
         extern __shared__ __align__(128) unsigned char smem[];
         __shared__ uint64_t bar;
-        pdl_launch_dependents();
+        trigger_early(a);
         FineTile<T> F(r0, nslices, cap, smem, bid);
         const bool valid = F.row >= r0 && F.row < r1;
         const int len = valid ? (int)__ldcs(rlen + F.row) : 0;
         const T di = valid ? __ldcs(dinv + F.row) : T(0);
         if (!stage_tile(F, a, &bar)) return;
-        pdl_wait();
+        wait_and_trigger(a);
         if (!valid) return;
         const T xi = fine_row<T>(F, len, jmax, [&](int j) { return x[j]; }, b[F.row], a.n, a.err) * di;
         x[F.row] = xi;
@@ -1040,13 +1058,13 @@ struct FineResidualBody {
         T* r = static_cast<T*>(a.out);
         extern __shared__ __align__(128) unsigned char smem[];
         __shared__ uint64_t bar;
-        pdl_launch_dependents();
+        trigger_early(a);
         FineTile<T> F(r0, nslices, cap, smem, bid);
         const bool valid = F.row >= r0 && F.row < n;
         const int len = valid ? (int)__ldcs(rlen + F.row) : 0;
         const T dg = valid ? __ldcs(diag + F.row) : T(0);
         if (!stage_tile(F, a, &bar)) return;
-        pdl_wait();
+        wait_and_trigger(a);
         if (!valid) return;
         r[F.row] = fine_row<T>(F, len, n, [&](int j) { return x[j]; }, fmad(-dg, x[F.row], b[F.row]),
                                a.n, a.err);
@@ -1066,14 +1084,14 @@ struct FineSplitPassBody {
         T* sv = static_cast<T*>(a.out);
         extern __shared__ __align__(128) unsigned char smem[];
         __shared__ uint64_t bar;
-        pdl_launch_dependents();
+        trigger_early(a);
         FineTile<T> F(r0, a.nslices, a.cap, smem, bid);
         const bool valid = F.row >= r0 && F.row < r1;
         const int low = valid ? (int)a.rlow[F.row] : 0;
         const int up = (valid && PART != kPartLower) ? (int)a.rlen[F.row] - low : 0;
         const T di = valid ? dinv[F.row] : T(0);
         if (!stage_tile(F, a, &bar)) return;
-        pdl_wait();
+        wait_and_trigger(a);
         if (!valid) return;
         T s = b[F.row];
         if (PART != kPartUpper) s = fine_part<false, T>(F, low, x, s, a.n, a.err);
@@ -1094,12 +1112,12 @@ struct FineSplitResidualBody {
         T* r = static_cast<T*>(a.out);
         extern __shared__ __align__(128) unsigned char smem[];
         __shared__ uint64_t bar;
-        pdl_launch_dependents();
+        trigger_early(a);
         FineTile<T> F(r0, a.nslices, a.cap, smem, bid);
         const bool valid = F.row >= r0 && F.row < n;
         const int low = valid ? (int)a.rlow[F.row] : 0;
         if (!stage_tile(F, a, &bar)) return;
-        pdl_wait();
+        wait_and_trigger(a);
         if (!valid) return;
         r[F.row] = fine_part<false, T>(F, low, x, b[F.row] - r[F.row], a.n, a.err);
     }
@@ -1131,7 +1149,7 @@ struct FineResRestrictBody {
         __shared__ uint64_t bar;
         __shared__ T sv[kFineBlock];
         __shared__ int sk[kFineBlock];
-        pdl_launch_dependents();
+        trigger_early(a);
         FineTile<T> F(c1, nslices, cap, smem, bid);
         const bool valid = F.row >= c1 && F.row < n;
         const int len = valid ? (int)__ldcs(rlen + F.row) : 0;
@@ -1139,7 +1157,7 @@ struct FineResRestrictBody {
         const int key = valid ? __ldcs(agg + F.row) : -1;
         const T ti = (SCALED && valid) ? __ldcs(t + F.row) : T(1);
         if (!stage_tile(F, a, &bar)) return;
-        pdl_wait();
+        wait_and_trigger(a);
         T v = T(0);
         if (valid) {
             const T ri = fine_row<T>(F, len, n, [&](int j) { return x[j]; },
@@ -1171,14 +1189,14 @@ struct RestrictBody {
         const T* __restrict__ t = static_cast<const T*>(a.t);
         const T* r = static_cast<const T*>(a.b);
         T* bc = static_cast<T*>(a.out);
-        pdl_launch_dependents();
+        trigger_early(a);
         const int J = bid * blockDim.x + threadIdx.x;
         if (J >= nc) return;
         const int kb = rptr[J], k1 = rptr[J + 1];
         int i[kUnroll];
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) i[u] = (kb + u < k1) ? ridx[kb + u] : -1;
-        pdl_wait();
+        wait_and_trigger(a);
         T s = T(0);
         for (int k0 = kb; k0 < k1; k0 += kUnroll) {
             if (k0 > kb) {
@@ -1214,13 +1232,13 @@ struct ProlongBody {
         const T* e = static_cast<const T*>(a.b);
         T* x = static_cast<T*>(a.x);
         const T omega = (T)a.omega;
-        pdl_launch_dependents();
+        trigger_early(a);
         const int i = r0 + (int)(bid * blockDim.x + threadIdx.x);
         if (i >= n) return;
         const int g = agg[i];
         if (g < 0 || !index_ok(g, a.nc, a.err)) return;
         const T w = SCALED ? omega * t[i] : omega;
-        pdl_wait();
+        wait_and_trigger(a);
         x[i] = fmad(w, e[g], x[i]);
     }
 };
@@ -1241,14 +1259,14 @@ struct GemvBody {
         const TB* b = static_cast<const TB*>(a.b);
         TB* x = static_cast<TB*>(a.x);
         extern __shared__ double sbuf[];
-        pdl_launch_dependents();
+        trigger_early(a);
         const int lane = threadIdx.x & 31;
         const int row = (int)((bid * (int64_t)blockDim.x + threadIdx.x) >> 5);
         const double* m = M + (size_t)min(row, n - 1) * n;
         double m0[kPre];
 #pragma unroll
         for (int u = 0; u < kPre; ++u) m0[u] = (lane + 32 * u < n) ? m[lane + 32 * u] : 0.0;
-        pdl_wait();
+        wait_and_trigger(a);
         const double* sb;
         if (kStage) {
             for (int k = threadIdx.x; k < n; k += blockDim.x) sbuf[k] = (double)b[k];
@@ -1291,7 +1309,7 @@ struct GemvF32Body {
         const float* __restrict__ M = static_cast<const float*>(a.dv);
         const float* __restrict__ b = static_cast<const float*>(a.b);
         float* x = static_cast<float*>(a.x);
-        pdl_launch_dependents();
+        trigger_early(a);
         const int lane = threadIdx.x & 31;
         const int row = (int)((bid * (int64_t)blockDim.x + threadIdx.x) >> 5);
         const int q4 = ld >> 2;
@@ -1300,7 +1318,7 @@ struct GemvF32Body {
         float4 v[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) v[u] = lane + 32 * u < q4 ? m[lane + 32 * u] : zero;
-        pdl_wait();
+        wait_and_trigger(a);
         if (row >= n) return;
         float acc[kU] = {};
         for (int q = lane;; q += 32 * kU) {
@@ -1352,11 +1370,11 @@ struct ToScaledBody {
         const double* r = a.rin;
         const double* __restrict__ isq = a.isq;
         float* rhat = static_cast<float*>(a.x);
-        pdl_launch_dependents();
+        trigger_early(a);
         const int i = bid * blockDim.x + threadIdx.x;
         if (i >= n) return;
         const double w = isq[i];
-        pdl_wait();
+        wait_and_trigger(a);
         rhat[i] = (float)(r[i] * w);
     }
 };
@@ -1369,11 +1387,11 @@ struct FromScaledBody {
         const float* zhat = static_cast<const float*>(a.b);
         const double* __restrict__ isq = a.isq;
         double* z = a.z;
-        pdl_launch_dependents();
+        trigger_early(a);
         const int i = bid * blockDim.x + threadIdx.x;
         if (i >= n) return;
         const double w = isq[i];
-        pdl_wait();
+        wait_and_trigger(a);
         z[i] = (double)zhat[i] * w;
     }
 };
@@ -1890,9 +1908,10 @@ void vbatch_launch(const VRec* const* recs, int n, cudaStream_t s) {
         smem = std::max(smem, recs[k]->smem);
         if (recs[k]->carve != carve) carve = -1;
     }
+    for (int k = 0; k < n; ++k) p.a[k].late = p.bstart[n] > g_overlap_max_blocks;
     // the 48 KB default covers static and dynamic shared memory together
     if (smem > kDefaultDynSmem) raise_dyn_smem(k_batched<Body>, smem);
-    launch_kernel_carve(k_batched<Body>, p.bstart[n], recs[0]->block, smem, carve, s, p);
+    launch_kernel_carve(k_batched<Body>, p.bstart[n], recs[0]->block, smem, carve, true, s, p);
 }
 
 thread_local std::vector<VRec>* t_vrecord = nullptr;
@@ -1918,7 +1937,9 @@ void vlaunch(int grid, int block, size_t smem, cudaStream_t s, const VArgs& a, i
         return;
     }
     if (smem > kDefaultDynSmem) raise_dyn_smem(k_single<Body>, smem);
-    launch_kernel_carve(k_single<Body>, grid, block, smem, carve, s, a);
+    VArgs q = a;
+    q.late = grid > g_overlap_max_blocks;
+    launch_kernel_carve(k_single<Body>, grid, block, smem, carve, true, s, q);
 }
 
 // arguments shared by the row kernels of a level
