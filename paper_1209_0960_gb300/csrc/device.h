@@ -249,6 +249,10 @@ struct DevLevel {
     // W - 1, W - 2, ..., so a pass that needs one part reads whole lines of it
     bool split = false;
     uint16_t* rlow = nullptr;         // [n] entries towards earlier colours (split levels)
+    // split levels small enough for the tail (kTailMaxRows): running counts of
+    // the rows' entries, and of the members of the coarse rows' restriction lists
+    int32_t* nrp = nullptr;           // [n+1]
+    std::vector<int32_t> nrp_host, rptr_host;
     int32_t* scol = nullptr;          // [padded] permuted column indices
     double* sval = nullptr;           // [padded]
     // sliced layout with per-slice widths, for the staged kernels on levels
@@ -283,9 +287,16 @@ struct DevLevel {
     // pre-smoother (first two colours from zero, forward, backward) and the
     // post-smoother (forward, backward), planned for rows = block / lpr
     bool sweep = false;
+    // part of the tail: with every level below, run by the cluster kernel of
+    // tail.cu (levels of a few thousand rows; see tail_fits)
+    bool tail = false;
     const SweepPlan* plan_pre = nullptr;
     const SweepPlan* plan_post = nullptr;
 };
+
+// rows of a level of the tail (tail.cu) stay below this: its columns have 16
+// bits, and this value marks none
+constexpr int32_t kTailMaxRows = 65535;
 
 // largest tile of the staged kernels (index and value of the entries of 8
 // consecutive slices): two blocks still fit on an SM.  With the common width
@@ -588,9 +599,11 @@ void galerkin_device(const DevCsr& A, const HostCsr& Ah, const AggResult& agg, D
 
 // Build the smoothing-order device level from the original-order device
 // matrix A and the permutation perm (original -> new position).
-// split: store the rows split by colour (see DevLevel::split).
+// split: store the rows split by colour (see DevLevel::split); low then gets
+// the lengths of the lower parts.
 void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<int32_t>& perm,
-                        bool split, DevArena& arena, DevLevel& L, cudaStream_t s);
+                        bool split, DevArena& arena, DevLevel& L, std::vector<uint16_t>& low,
+                        cudaStream_t s);
 
 // Decoupled aggregation (Alg. 4) on the device: the rows of A (original
 // order) split into consecutive tiles of p.aggregation_tile rows, one warp per
@@ -612,6 +625,21 @@ void scale_inverse_device(int n, const double* diag, const double* Minv, double*
 // coarse neighbour (for t32); coarse_diag is null on the coarsest level.
 void build_level_fp32(DevLevel& L, const double* coarse_diag, DevArena& arena, cudaStream_t s);
 
+}  // namespace amg
+
+namespace amg {
+// The tail of the V-cycle (tail.cu): everything from one level down as one
+// launch, or as two around the coarsest solve where that is too large for the
+// cluster's SMs.
+struct TailHalf {
+    void* desc = nullptr;     // device descriptor
+    size_t smem = 0;          // shared memory per block
+    int blocks = 0;           // blocks of the cluster
+};
+struct Tail {
+    bool one = true;          // down covers the whole V-cycle from the level
+    TailHalf down, up;
+};
 }  // namespace amg
 
 // State of a CG solve driven one step at a time (pcg_async_*).
@@ -647,6 +675,8 @@ struct amg_ctx {
     int32_t last_device_loop = 0;         // the last PCG solve ran its loop on the device
     bool use_graphs = true;
     amg::DevArena mem;
+    std::map<int, amg::Tail> tails[2];    // by first level, float64 and float32
+    int tail_l0 = 0x7fffffff;             // first level of the tail with the current shapes
     std::vector<amg::HostLevel> hl;
     std::vector<amg::DevLevel> dl;
     int32_t nL = 0;                   // coarsest size
@@ -720,6 +750,13 @@ struct amg_ctx {
 };
 
 namespace amg {
+// whether the levels from l0 down can run as a tail
+bool tail_fits(const amg_ctx* c, int l0, bool f32);
+// the tail from level l0, built on first use (not while a stream is captured)
+const Tail& tail_of(amg_ctx* c, int l0, bool f32);
+// one launch of the tail, or its record while a V-cycle is being recorded
+void launch_tail(const TailHalf& h, bool f32, cudaStream_t s);
+
 // CG driven one step at a time on a context's own stream (solver.cu); the
 // launches, and so the results, are those of amg_pcg_solve.  begin expects the
 // right-hand side in c->bb and the initial guess in c->x (smoothing order).

@@ -519,7 +519,8 @@ void galerkin_device(const DevCsr& A, const HostCsr& Ah, const AggResult& R, Dev
 }
 
 void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<int32_t>& perm,
-                        bool split, DevArena& arena, DevLevel& L, cudaStream_t s) {
+                        bool split, DevArena& arena, DevLevel& L, std::vector<uint16_t>& low,
+                        cudaStream_t s) {
     const int32_t n = Ah.n;
     std::vector<int32_t> inv(n), nrp(n + 1, 0);
     std::vector<uint16_t> rlen(n);
@@ -570,7 +571,8 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
     DevArena tmp(s);
     int32_t* d_inv = tmp.alloc<int32_t>(n);
     int32_t* d_perm = tmp.alloc<int32_t>(n);
-    int32_t* d_nrp = tmp.alloc<int32_t>(n + 1);
+    const bool keep_nrp = split && n < kTailMaxRows;
+    int32_t* d_nrp = (keep_nrp ? arena : tmp).alloc<int32_t>(n + 1);
     int32_t* d_nci = tmp.alloc<int32_t>(L.nnz_off);
     double* d_nva = tmp.alloc<double>(L.nnz_off);
     AMG_CUDA_TRY(cudaMemcpyAsync(d_inv, inv.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s));
@@ -613,6 +615,16 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
         L.lpr = (avg <= 7.0 && staged_fits(L)) ? 0 : avg <= 16.0 ? 4 : 8;
     }
     L.lpr_wide = L.lpr;
+    if (keep_nrp) {
+        L.nrp = d_nrp;
+        L.nrp_host = nrp;
+    }
+    // entries of each colour's lower parts (the colours' first rows are known
+    // to the caller only: it sums low over them)
+    if (split) {
+        low.resize(n);
+        AMG_CUDA_TRY(cudaMemcpyAsync(low.data(), L.rlow, sizeof(uint16_t) * n, cudaMemcpyDeviceToHost, s));
+    }
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
 }
 

@@ -334,6 +334,41 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
         k_coarsest(c, b, x);
         return;
     }
+    if (l >= c->tail_l0) {
+        // this level and all below as one cluster launch (two around the
+        // coarsest solve where that runs over all SMs)
+        const Tail& t = tail_of(c, l, scaled);
+        double down = 0.0, up = 0.0;
+        for (int k = l; k < nlev - 1; ++k) {
+            const DevLevel& K = c->dl[k];
+            const int C = K.ncolours;
+            down += first_bytes(K, vb) + residual_restrict_bytes(K, vb, scaled);
+            up += prolong_bytes(K, vb, scaled);
+            for (int col = 2; col < C; ++col) down += pass_bytes(K, col, K.cptr[col], vb, kPartLower);
+            for (int col = 0; col < C; ++col) up += pass_bytes(K, col, K.n, vb);
+            for (int col = C - 2; col >= 0; --col) {
+                down += pass_bytes(K, col, K.n, vb, kPartUpper);
+                up += pass_bytes(K, col, K.n, vb, kPartUpper);
+            }
+        }
+        if (t.one) {
+            const double mb = (vb == 4 && c->Ainv_s32) ? 4.0 : 8.0;
+            ProfScope ps(c, kKCoarseSolve, down + up + (double)c->nL * c->nL * mb + 2.0 * vb * c->nL);
+            vkey(0, l, 0);
+            launch_tail(t.down, scaled, s);
+            return;
+        }
+        {
+            ProfScope ps(c, kKGsCoarse, down);
+            vkey(0, l, 0);
+            launch_tail(t.down, scaled, s);
+        }
+        vcycle<T>(c, nlev - 1, P::b(c->dl[nlev - 1]), P::x(c->dl[nlev - 1]));
+        ProfScope ps(c, kKGsCoarse, up);
+        vkey(1, 64 - l, 0);
+        launch_tail(t.up, scaled, s);
+        return;
+    }
     DevLevel& N = c->dl[l + 1];
     const int C = L.ncolours;
     const int kind = l == 0 ? kKGsL0 : kKGsCoarse;
@@ -554,10 +589,13 @@ constexpr int kStaged = 0;   // DevLevel::lpr of the staged one-row-per-thread k
 // A launch shape as one code: lanes per row (0 = staged kernels, 1, 2, 4 or
 // 8) plus kHalfBlock for blocks of 128 instead of 256 threads (row kernels
 // only), plus kSweep for smoothing sweeps run as one dependency-driven kernel
-// each (lane shapes only), plus (staged kernels only) the preferred
-// shared-memory carveout + 1 in the bits from kCarveShift (0: the driver's).
+// each (lane shapes only), plus kTail for a level that joins the tail when all
+// levels below do (split levels; the lanes then serve only as the shape outside
+// the tail), plus (staged kernels only) the preferred shared-memory carveout + 1
+// in the bits from kCarveShift (0: the driver's).
 constexpr int kHalfBlock = 16;
 constexpr int kSweep = 32;
+constexpr int kTail = 64;
 constexpr int kCarveShift = 8;
 constexpr int kCarveMask = 0x7f << kCarveShift;
 // sweeps are planned on the host from the level's graph (adjacency of every
@@ -570,6 +608,7 @@ inline int with_carve(int code, int carve) { return (code & ~kCarveMask) | ((car
 
 bool shape_allowed(const DevLevel& L, int code) {
     const int lanes = shape_lanes(code);
+    if (code & kTail) return L.split && !(code & kSweep) && shape_allowed(L, code & ~kTail);
     if (code & ~(kSweep | kHalfBlock | (kHalfBlock - 1) | kCarveMask)) return false;
     if (shape_carve(code) > 100) return false;
     if (lanes == kStaged) return (code & ~kCarveMask) == kStaged && staged_fits(L);
@@ -582,7 +621,8 @@ bool shape_allowed(const DevLevel& L, int code) {
 }
 
 int shape_of(const DevLevel& L) {
-    const int code = L.lpr | (L.block == 128 ? kHalfBlock : 0) | (L.sweep ? kSweep : 0);
+    const int code = L.lpr | (L.block == 128 ? kHalfBlock : 0) | (L.sweep ? kSweep : 0) |
+                     (L.tail ? kTail : 0);
     return L.lpr == kStaged && L.carve >= 0 ? with_carve(code, L.carve) : code;
 }
 
@@ -692,6 +732,29 @@ void plan_sweep(amg_ctx* c, int l, int rows, bool pre, SweepPlan& P) {
     AMG_CUDA_TRY(cudaStreamSynchronize(s));   // the host vectors go out of scope
 }
 
+// Levels that join the tail without being timed: in float64, where 16 SMs run
+// the arithmetic of a pass at a tenth of the device's rate, up to about 7,000
+// rows (6,619 rows: 69.8 us from the level against 73.8 as launches; 13,113
+// rows: 132 against 75 before the entries moved to shared memory); in float32
+// as far as the tail fits in shared memory (about 18,000 rows).
+inline bool tail_rule(const DevLevel& L, bool f32) { return L.split && (f32 || L.n <= 7000); }
+
+// The first level of the tail under the levels' current shapes, and its
+// descriptors (built here: V-cycles are captured into graphs).  Called after
+// set_shape.
+void find_tail(amg_ctx* c) {
+    const bool f32 = c->precision == AMG_FP32_IN_FP64;
+    const int nlev = (int)c->dl.size();
+    c->tail_l0 = nlev;
+    while (c->tail_l0 > 1 && c->tail_l0 - 1 < nlev) {
+        const int l = c->tail_l0 - 1;
+        if (l < nlev - 1 && !(c->dl[l].tail && tail_fits(c, l, f32))) break;
+        c->tail_l0 = l;
+    }
+    if (c->tail_l0 >= nlev - 1) c->tail_l0 = nlev;   // the coarsest level alone is no tail
+    if (c->tail_l0 < nlev) tail_of(c, c->tail_l0, f32);
+}
+
 void set_shape(amg_ctx* c, int l, int code) {
     DevLevel& L = c->dl[l];
     const int lanes = shape_lanes(code);
@@ -701,6 +764,7 @@ void set_shape(amg_ctx* c, int l, int code) {
     L.fused_restrict = lanes == kStaged && L.fused_ok;
     L.sweep = (code & kSweep) != 0 && lanes >= 1;
     L.carve = lanes == kStaged ? shape_carve(code) : -1;
+    L.tail = (code & kTail) != 0;
     L.plan_pre = L.plan_post = nullptr;
     if (L.sweep) {
         // the plan (items, and the cooperative grid) depends on lanes and block
@@ -742,6 +806,7 @@ std::map<ShapeKey, int> g_shape_cache;
 // sized to about 0.3 ms each.
 double time_vcycle_from(amg_ctx* c, int l) {
     cudaStream_t s = c->stream;
+    if (l >= c->tail_l0) tail_of(c, l, c->precision == AMG_FP32_IN_FP64);
     cudaGraphExec_t g = capture_graph(c, [&] {
         if (l == 0) precondition(c, c->r, c->z);
         else if (c->precision == AMG_FP64) vcycle64(c, l, c->dl[l].b, c->dl[l].x);
@@ -798,6 +863,7 @@ double autotune_shapes(amg_ctx* c) {
             auto it = g_shape_cache.find(key);
             if (it != g_shape_cache.end() && shape_allowed(L, it->second)) {
                 set_shape(c, l, it->second);
+                find_tail(c);
                 continue;
             }
         }
@@ -805,18 +871,25 @@ double autotune_shapes(amg_ctx* c) {
             zero_inputs();
             timed = true;
         }
-        const int rule = L.lpr;
+        const int rule = shape_of(L);
         double t_rule = 1e30, t_best = 1e30;
         int best = rule;
         // staged kernels also with a smaller shared-memory carveout (percent
         // of the maximum 228 KB: 100, 132 or 164 KB), leaving more L1 for the
         // neighbour gathers
-        for (int lanes : {kStaged, with_carve(kStaged, 44), with_carve(kStaged, 58),
-                          with_carve(kStaged, 72), 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4,
-                          4 | kHalfBlock, 8, 8 | kHalfBlock, 2 | kSweep, 2 | kHalfBlock | kSweep,
-                          4 | kSweep, 4 | kHalfBlock | kSweep, 8 | kSweep, 8 | kHalfBlock | kSweep}) {
+        std::vector<int> tries = {kStaged, with_carve(kStaged, 44), with_carve(kStaged, 58),
+                                  with_carve(kStaged, 72), 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4,
+                                  4 | kHalfBlock, 8, 8 | kHalfBlock, 2 | kSweep,
+                                  2 | kHalfBlock | kSweep, 4 | kSweep, 4 | kHalfBlock | kSweep,
+                                  8 | kSweep, 8 | kHalfBlock | kSweep};
+        // the tail, where every level below is in it
+        if (L.split && (l == nlev - 2 || c->tail_l0 <= l + 1) &&
+            tail_fits(c, l, c->precision == AMG_FP32_IN_FP64))
+            tries.push_back(rule | kTail);
+        for (int lanes : tries) {
             if (!shape_allowed(L, lanes)) continue;
             set_shape(c, l, lanes);
+            find_tail(c);
             const double t = time_vcycle_from(c, l);
             if (lanes == rule) t_rule = t;
             if (t < t_best) {
@@ -830,6 +903,7 @@ double autotune_shapes(amg_ctx* c) {
         std::lock_guard<std::mutex> lk(g_shape_mu);
         const int stored = g_shape_cache.emplace(key, best).first->second;
         set_shape(c, l, shape_allowed(L, stored) ? stored : best);
+        find_tail(c);
     }
     for (int l = 0; l + 1 < nlev; ++l) c->shapes[c->precision][l] = shape_of(c->dl[l]);
     c->tuned[c->precision] = true;
@@ -841,6 +915,7 @@ double autotune_shapes(amg_ctx* c) {
 // Make the levels run the shapes of the context's precision.
 void apply_shapes(amg_ctx* c) {
     for (int l = 0; l + 1 < (int)c->dl.size(); ++l) set_shape(c, l, c->shapes[c->precision][l]);
+    find_tail(c);
 }
 
 // ---------------------------------------------------------------------------
@@ -1099,6 +1174,8 @@ int pcg(amg_ctx* c, double tol, int32_t maxit, amg_solve_info* info) {
             auto& gv = c->graph_from[c->precision];
             gv.resize(c->dl.size(), nullptr);
             for (int l = 1; l < (int)c->dl.size(); ++l) {
+                if (l >= c->tail_l0 && l < (int)c->dl.size() - 1)
+                    tail_of(c, l, c->precision == AMG_FP32_IN_FP64);
                 if (!gv[l])
                     gv[l] = capture_graph(c, [&] {
                         if (c->precision == AMG_FP64) vcycle64(c, l, c->dl[l].b, c->dl[l].x);
@@ -1629,7 +1706,8 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     for (int l = 0; l < nlev; ++l) {
         HostLevel& h = c->hl[l];
         DevLevel& L = c->dl[l];
-        build_level_device(dA[l], h.A, h.perm, l > 0 && l < nlev - 1 && h.ncolours >= 3, c->mem, L, s);
+        std::vector<uint16_t> low;
+        build_level_device(dA[l], h.A, h.perm, l > 0 && l < nlev - 1 && h.ncolours >= 3, c->mem, L, low, s);
         L.x = c->mem.alloc<double>(L.n);
         L.b = c->mem.alloc<double>(L.n);
         L.r = c->mem.alloc<double>(L.n);
@@ -1647,10 +1725,6 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
         }
         for (int col = 0; col < h.ncolours; ++col) L.cptr[col + 1] += L.cptr[col];
         if (L.split) {
-            std::vector<uint16_t> low(L.n);
-            AMG_CUDA_TRY(cudaMemcpyAsync(low.data(), L.rlow, sizeof(uint16_t) * L.n,
-                                         cudaMemcpyDeviceToHost, s));
-            AMG_CUDA_TRY(cudaStreamSynchronize(s));
             L.clow.assign(h.ncolours, 0);
             for (int col = 0; col < h.ncolours; ++col)
                 for (int32_t r = L.cptr[col]; r < L.cptr[col + 1]; ++r) L.clow[col] += low[r];
@@ -1688,6 +1762,7 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
         upload(L.agg, aggp, s);
         upload(L.rptr, rptr, s);
         upload(L.ridx, ridx, s);
+        if (L.nrp) L.rptr_host = rptr;
     }
     // coarsest level: dense inverse
     c->Ainv = c->mem.alloc<double>((size_t)c->nL * c->nL);
@@ -1743,8 +1818,10 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     if (c->precision == AMG_FP32_IN_FP64) ensure_fp32(c.get());
     for (int pr = 0; pr < 2; ++pr) {
         c->shapes[pr].assign(nlev - 1, 0);
-        for (int l = 0; l + 1 < nlev; ++l) c->shapes[pr][l] = shape_of(c->dl[l]);
+        for (int l = 0; l + 1 < nlev; ++l)
+            c->shapes[pr][l] = shape_of(c->dl[l]) | (tail_rule(c->dl[l], pr == AMG_FP32_IN_FP64) ? kTail : 0);
     }
+    apply_shapes(c.get());
     const double tune_ms = prm->autotune ? autotune_shapes(c.get()) : 0.0;
     fill_info(c.get());
     c->summary.autotune_ms = tune_ms;
@@ -2001,6 +2078,7 @@ int amg_set_level_shape(amg_ctx* c, int32_t l, int32_t lanes_per_row, int32_t th
         AMG_CUDA_TRY(cudaStreamSynchronize(c->stream));   // no graph of this context in flight
         drop_graphs(c);
         set_shape(c, l, code);
+        find_tail(c);
         c->shapes[c->precision][l] = code;
         c->linfo[l].lanes_per_row = c->dl[l].lpr;
         c->linfo[l].threads_per_block = c->dl[l].block;
@@ -2023,6 +2101,7 @@ int amg_set_level_carveout(amg_ctx* c, int32_t l, int32_t percent) {
         drop_graphs(c);
         const int code = with_carve(shape_of(c->dl[l]), percent);
         set_shape(c, l, code);
+        find_tail(c);
         c->shapes[c->precision][l] = code;
         c->linfo[l].carveout = c->dl[l].carve;
         leave(c);
@@ -2163,6 +2242,10 @@ int amg_debug_set_column(amg_ctx* c, int32_t l, int32_t row, int32_t k, int32_t 
             AMG_CUDA_TRY(cudaMemcpy(L.ccol + pos, &col, sizeof(int32_t), cudaMemcpyHostToDevice));
         }
         drop_graphs(c);
+        // the tail's packed copy of the entries
+        c->tails[0].clear();
+        c->tails[1].clear();
+        find_tail(c);
 #endif
     });
 }
