@@ -55,6 +55,100 @@ __device__ __forceinline__ T sell_row(int64_t base, int len, const int32_t* __re
     return acc;
 }
 
+// One row of a level whose slices are W entries wide, held by its thread: with
+// the width a constant, all entries of the row are loaded at once and all its
+// gathers follow at once, two round trips to memory per row.  (A loop over the
+// row's length took a round trip for the length and two for each batch of
+// four entries.)  Slots past the row's length are padding whose column is the
+// row itself; their values are not used.
+template <typename T, int W>
+struct WideRow {
+    int j[W];
+    T a[W], d;
+    int len;
+    __device__ __forceinline__ void load(int row, bool in, int64_t sw, const uint16_t* __restrict__ rlen,
+                                         const int32_t* __restrict__ scol,
+                                         const T* __restrict__ sval, const T* __restrict__ dv) {
+        const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
+        len = in ? (int)__ldcs(rlen + row) : 0;
+        d = in ? __ldcs(dv + row) : T(0);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            j[k] = in ? __ldcs(scol + base + 32 * k) : 0;
+            a[k] = in ? __ldcs(sval + base + 32 * k) : T(0);
+        }
+    }
+    // acc +- sum over the entries (ALL, or those with j < jmax) of a x_j, in
+    // stored order
+    template <bool NEG, bool ALL>
+    __device__ __forceinline__ T add(const T* x, T acc, int jmax, int n, int32_t* err) const {
+        T v[W];
+#pragma unroll
+        for (int k = 0; k < W; ++k) v[k] = (!kChecks || (k < len && index_ok(j[k], n, err))) ? x[j[k]] : T(0);
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if (k < len && (ALL || j[k] < jmax)) acc = fmad(NEG ? -a[k] : a[k], v[k], acc);
+        return acc;
+    }
+};
+
+// The rows of a CG kernel, a thread per row, grid-stride: start(row, A_ii) is
+// the value a row's sum starts from, done(row, value) takes it.  With the slice
+// width W a constant the next row's entries are loaded while the current row is
+// summed (the first row's before the caller waits for the kernel before it),
+// in four blocks per SM: 51.2 -> 41.7 us for q = A p on 2.1M rows and 245 -> 205
+// us on 12M, against the loop over sell_row in eight (without the prefetch 47.1
+// and 217; three blocks per SM 42.7 and 226).
+template <int W>
+struct RowLoop {
+    int n;
+    int64_t sw;
+    const uint16_t* __restrict__ rlen;
+    const int32_t* __restrict__ scol;
+    const double* __restrict__ sval;
+    const double* __restrict__ diag;
+    WideRow<double, W> cur;
+    int row, step;
+    __device__ __forceinline__ RowLoop(int n_, int64_t sw_, const uint16_t* rlen_, const int32_t* scol_,
+                                       const double* sval_, const double* diag_)
+        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_),
+          row(blockIdx.x * blockDim.x + threadIdx.x), step(gridDim.x * blockDim.x) {
+        cur.load(row, row < n, sw, rlen, scol, sval, diag);
+    }
+    template <bool NEG, typename Start, typename Done>
+    __device__ __forceinline__ void run(const double* x, int32_t* err, Start start, Done done) {
+        while (row < n) {
+            const int64_t after = (int64_t)row + step;
+            WideRow<double, W> next;
+            next.load((int)(after < n ? after : 0), after < n, sw, rlen, scol, sval, diag);
+            done(row, cur.template add<NEG, true>(x, start(row, cur.d), n, n, err));
+            if (after >= n) break;
+            row = (int)after;
+            cur = next;
+        }
+    }
+};
+template <>
+struct RowLoop<0> {
+    int n;
+    int64_t sw;
+    const uint16_t* __restrict__ rlen;
+    const int32_t* __restrict__ scol;
+    const double* __restrict__ sval;
+    const double* __restrict__ diag;
+    __device__ __forceinline__ RowLoop(int n_, int64_t sw_, const uint16_t* rlen_, const int32_t* scol_,
+                                       const double* sval_, const double* diag_)
+        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_) {}
+    template <bool NEG, typename Start, typename Done>
+    __device__ __forceinline__ void run(const double* x, int32_t* err, Start start, Done done) {
+        for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
+            const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
+            done(row, sell_row<NEG>(base, __ldcs(rlen + row), scol, sval, x, start(row, __ldcs(diag + row)),
+                                    n, err));
+        }
+    }
+};
+
 __device__ __forceinline__ double block_sum(double v, double* sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -1085,15 +1179,31 @@ struct FineSplitResidualBody {
     }
 };
 
+// Adds the sum of the values v of each run of equal keys in the warp (key -1:
+// none; equal keys are consecutive lanes) to bc[key].  Doubling steps, as many
+// as the longest run needs: two or three float64 additions a warp where a walk
+// along the run took one per row.
+template <typename T>
+__device__ __forceinline__ void restrict_runs(T v, int key, T* bc) {
+    const int lane = threadIdx.x & 31;
+    const int before = __shfl_up_sync(0xffffffffu, key, 1);
+    for (int off = 1; off < 32; off <<= 1) {
+        const bool same = __shfl_down_sync(0xffffffffu, key, off) == key && lane + off < 32 && key >= 0;
+        if (!__any_sync(0xffffffffu, same)) break;
+        const T w = __shfl_down_sync(0xffffffffu, v, off);
+        if (same) v += w;
+    }
+    if (key >= 0 && (lane == 0 || before != key)) atomicAdd(bc + key, v);
+}
+
 // Residual and restriction in one pass on a two-colour fine level: the rows
 // of colour 1 ([c1, n)) are sorted by coarse index, so the rows of one
 // aggregate are consecutive (with more colours an aggregate would recur in
-// every colour block).  Each thread stores (t_i) r_i in shared memory; the
-// first row of every run of equal coarse index inside the block sums the run
-// in order and adds it to bc (zeroed by the first pass).  A run is shorter
-// than a block, so a coarse entry receives at most two additions onto zero (a
-// run cut by a block boundary), whose result does not depend on their order:
-// the sum stays deterministic.  Arguments: r0 = c1, r1 = n, width, nslices,
+// every colour block).  Each run of equal coarse index inside a warp is summed
+// and added to bc (zeroed by the first pass).  A run is at most 32 rows, so a
+// coarse entry receives at most two additions onto zero (a run cut by a warp
+// boundary), whose result does not depend on their order: the sum stays
+// deterministic.  Arguments: r0 = c1, r1 = n, width, nslices,
 // cap, soff, dv = A_ii, idx = aggregate map, t, out = bc, err.
 template <typename T, bool SCALED>
 struct FineResRestrictBody {
@@ -1109,8 +1219,6 @@ struct FineResRestrictBody {
         T* bc = static_cast<T*>(a.out);
         extern __shared__ __align__(128) unsigned char smem[];
         __shared__ uint64_t bar;
-        __shared__ T sv[kFineBlock];
-        __shared__ int sk[kFineBlock];
         trigger_early(a);
         FineTile<T> F(c1, nslices, cap, smem, bid);
         const bool valid = F.row >= c1 && F.row < n;
@@ -1126,14 +1234,60 @@ struct FineResRestrictBody {
                                      fmad(-dg, x[F.row], b[F.row]), a.n, a.err);
             v = SCALED ? ti * ri : ri;
         }
-        const int tid = threadIdx.x;
-        sv[tid] = v;
-        sk[tid] = key;
-        __syncthreads();
-        if (key < 0 || (tid > 0 && sk[tid - 1] == key)) return;
-        T sum = v;
-        for (int u = tid + 1; u < kFineBlock && sk[u] == key; ++u) sum += sv[u];
-        atomicAdd(bc + key, sum);
+        restrict_runs(v, key, bc);
+    }
+};
+
+// The colour pass and the residual-restriction of a two-colour level whose
+// slices are W wide (the fine level of a 5-point or 7-point stencil), read
+// straight into registers (WideRow), a thread per row.  Against the staged
+// kernels, which copy the slices to shared memory, wait, and gather four
+// neighbours at a time, a pass has one wait fewer and all its gathers in flight:
+// 25.7 -> 21.8 us for a float64 pass over 1.05M rows, 45.7 -> 37.5 us over 2.2M,
+// 81.8 -> 73.0 us for a float32 pass over 6.0M.  (A persistent grid that loads
+// the next row ahead was slower here: 22.4, 39.4 and 79.9 us.)  Arguments as
+// FinePassBody and FineResRestrictBody.
+template <typename T, int W>
+struct WidePassBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int r0 = a.r0, r1 = a.r1;
+        const T* b = static_cast<const T*>(a.b);
+        T* x = static_cast<T*>(a.x);
+        trigger_early(a);
+        const int row = (r0 & ~31) + bid * kFineBlock + (int)threadIdx.x;
+        const bool valid = row >= r0 && row < r1;
+        WideRow<T, W> R;
+        R.load(valid ? row : r0, valid, a.sw, a.rlen, a.scol, static_cast<const T*>(a.sval),
+               static_cast<const T*>(a.dv));
+        wait_and_trigger(a);
+        if (!valid) return;
+        const T xi = R.template add<true, false>(x, b[row], a.jmax, a.n, a.err) * R.d;
+        x[row] = xi;
+        if (a.z) a.z[row] = (double)xi * a.isq[row];
+    }
+};
+
+template <typename T, bool SCALED, int W>
+struct WideResRestrictBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const int c1 = a.r0, n = a.r1;
+        const T* b = static_cast<const T*>(a.b);
+        const T* x = static_cast<const T*>(a.x);
+        trigger_early(a);
+        const int row = (c1 & ~31) + bid * kFineBlock + (int)threadIdx.x;
+        const bool valid = row >= c1 && row < n;
+        WideRow<T, W> R;
+        R.load(valid ? row : c1, valid, a.sw, a.rlen, a.scol, static_cast<const T*>(a.sval),
+               static_cast<const T*>(a.dv));
+        const int key = valid ? __ldcs(a.idx + row) : -1;
+        const T ti = (SCALED && valid) ? __ldcs(static_cast<const T*>(a.t) + row) : T(1);
+        wait_and_trigger(a);
+        T v = T(0);
+        if (valid) {
+            const T ri = R.template add<true, true>(x, fmad(-R.d, x[row], b[row]), n, a.n, a.err);
+            v = SCALED ? ti * ri : ri;
+        }
+        restrict_runs(v, key, static_cast<T*>(a.out));
     }
 };
 
@@ -1388,7 +1542,8 @@ __global__ void __launch_bounds__(kBlock) k_batched(const VBatch p) {
 // CG kernels (level 0, float64, smoothing order)
 // ---------------------------------------------------------------------------
 
-// r = b - A x and ||r||^2 (grid-stride over rows)
+// r = b - A x and ||r||^2 (grid-stride over rows; W: see RowLoop)
+template <int W>
 __global__ void __launch_bounds__(kBlock) k_cg_residual(int n, int64_t sw,
                                                         const uint16_t* __restrict__ rlen,
                                                         const int32_t* __restrict__ scol,
@@ -1401,20 +1556,21 @@ __global__ void __launch_bounds__(kBlock) k_cg_residual(int n, int64_t sw,
                                                         double* out, int mode) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
+    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
     pdl_wait();
     double acc = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
-        const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
-        const double s0 = fmad(-__ldcs(diag + row), x[row], b[row]);
-        const double v = sell_row<true>(base, __ldcs(rlen + row), scol, sval, x, s0, n, &sc->status);
-        if (r) r[row] = v;
-        acc = fmad(v, v, acc);
-    }
+    rows.template run<true>(
+        x, &sc->status, [&](int row, double d) { return fmad(-d, x[row], b[row]); },
+        [&](int row, double v) {
+            if (r) r[row] = v;
+            acc = fmad(v, v, acc);
+        });
     const double t = block_sum(acc, sh);
     finish_reduction(t, 0.0, partials, nullptr, counter, sc, out, mode, sh);
 }
 
 // q = A p and p.q -> alpha
+template <int W>
 __global__ void __launch_bounds__(kBlock) k_cg_spmv_pq(int n, int64_t sw,
                                                        const uint16_t* __restrict__ rlen,
                                                        const int32_t* __restrict__ scol,
@@ -1425,16 +1581,19 @@ __global__ void __launch_bounds__(kBlock) k_cg_spmv_pq(int n, int64_t sw,
                                                        unsigned int* counter, PcgScalars* sc) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
+    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
     pdl_wait();
-    double acc = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
-        const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
-        const double pi = p[row];
-        const double v = sell_row<false>(base, __ldcs(rlen + row), scol, sval, p,
-                                         __ldcs(diag + row) * pi, n, &sc->status);
-        q[row] = v;
-        acc = fmad(pi, v, acc);
-    }
+    double acc = 0.0, pi = 0.0;
+    rows.template run<false>(
+        p, &sc->status,
+        [&](int row, double d) {
+            pi = p[row];
+            return d * pi;
+        },
+        [&](int row, double v) {
+            q[row] = v;
+            acc = fmad(pi, v, acc);
+        });
     const double t = block_sum(acc, sh);
     finish_reduction(t, 0.0, partials, nullptr, counter, sc, nullptr, kPQ, sh);
 }
@@ -1642,6 +1801,7 @@ __device__ void finish_bi(double v0, double v1, double* partials, double* partia
 }
 
 // r = b - A x, rt = r, and the start scalars from r.r
+template <int W>
 __global__ void __launch_bounds__(kBlock) k_bi_start(int n, int64_t sw,
                                                      const uint16_t* __restrict__ rlen,
                                                      const int32_t* __restrict__ scol,
@@ -1652,16 +1812,16 @@ __global__ void __launch_bounds__(kBlock) k_bi_start(int n, int64_t sw,
                                                      unsigned int* counter, BiScalars* bs) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
+    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
     pdl_wait();
     double a = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
-        const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
-        const double s0 = fmad(-__ldcs(diag + row), x[row], b[row]);
-        const double v = sell_row<true>(base, __ldcs(rlen + row), scol, sval, x, s0, n, &bs->status);
-        r[row] = v;
-        rt[row] = v;
-        a = fmad(v, v, a);
-    }
+    rows.template run<true>(
+        x, &bs->status, [&](int row, double d) { return fmad(-d, x[row], b[row]); },
+        [&](int row, double v) {
+            r[row] = v;
+            rt[row] = v;
+            a = fmad(v, v, a);
+        });
     const double ta = block_sum(a, sh);
     finish_bi(ta, 0.0, partials, partials2, counter, bs, kBiStart, sh);
 }
@@ -1682,6 +1842,7 @@ __global__ void __launch_bounds__(kBlock) k_bi_direction(int n, const double* r,
 
 // y = A x with the dot products of the mode: kBiRtv: rt.y; kBiW: s.y and y.y
 // (skipped once the iteration has stopped)
+template <int W>
 __global__ void __launch_bounds__(kBlock) k_bi_spmv(int n, int64_t sw,
                                                     const uint16_t* __restrict__ rlen,
                                                     const int32_t* __restrict__ scol,
@@ -1692,17 +1853,17 @@ __global__ void __launch_bounds__(kBlock) k_bi_spmv(int n, int64_t sw,
                                                     unsigned int* counter, BiScalars* bs, int mode) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
+    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
     pdl_wait();
     if (bs->status || (mode == kBiW && bs->half)) return;
     double a = 0.0, b = 0.0;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
-        const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
-        const double v = sell_row<false>(base, __ldcs(rlen + row), scol, sval, x,
-                                         __ldcs(diag + row) * x[row], n, &bs->status);
-        y[row] = v;
-        a = fmad(w[row], v, a);
-        if (mode == kBiW) b = fmad(v, v, b);
-    }
+    rows.template run<false>(
+        x, &bs->status, [&](int row, double d) { return d * x[row]; },
+        [&](int row, double v) {
+            y[row] = v;
+            a = fmad(w[row], v, a);
+            if (mode == kBiW) b = fmad(v, v, b);
+        });
     const double ta = block_sum(a, sh);
     const double tb = block_sum(b, sh);
     finish_bi(ta, tb, partials, partials2, counter, bs, mode, sh);
@@ -1809,6 +1970,20 @@ inline int row_blocks(int r0, int r1, int lpr, int block = kBlock) {
 // latency, which more lanes per row shorten
 inline int launch_lpr(const DevLevel& L, int rows) {
     return rows >= L.wide_rows ? L.lpr_wide : L.lpr;
+}
+
+// the slice widths with kernels of their own: the 5-point and 7-point stencils
+#define AMG_WIDTH_DISPATCH(width, CALL)              \
+    switch (width) {                                 \
+        case 4: { constexpr int W = 4; CALL; } break;  \
+        case 6: { constexpr int W = 6; CALL; } break;  \
+        default: { constexpr int W = 0; CALL; } break; \
+    }
+inline bool wide_rows(int width) { return width == 4 || width == 6; }
+// grid of a CG kernel over rows: four blocks per SM with RowLoop<W > 0>, else eight
+inline int row_loop_blocks(const DevLevel& L) {
+    const int b = reduction_blocks(L.n);
+    return wide_rows(L.width) ? std::min(b, std::max(1, g_reduction_blocks / 2)) : b;
 }
 
 #define AMG_LPR_DISPATCH(lpr, CALL)                          \
@@ -1930,6 +2105,22 @@ void use_compact(const DevLevel& L, const LevelArrays<T>& A, VArgs& a) {
     a.sval = A.cval;
 }
 
+// levels of the staged kernels (lanes per row 0) that WideRow covers
+inline bool wide_level(const DevLevel& L) { return !L.split && !L.soff && wide_rows(L.width); }
+
+// one colour pass of a level that is not split, by the one-row-per-thread kernels
+template <typename T>
+void fine_pass(const DevLevel& L, const LevelArrays<T>& A, VArgs& a, cudaStream_t s) {
+    const int grid = fine_blocks(a.r0, a.r1);
+    if (wide_level(L)) {
+        if (L.width == 4) vlaunch<WidePassBody<T, 4>>(grid, kFineBlock, 0, s, a);
+        else vlaunch<WidePassBody<T, 6>>(grid, kFineBlock, 0, s, a);
+        return;
+    }
+    use_compact(L, A, a);
+    vlaunch<FinePassBody<T>>(grid, kFineBlock, fine_smem(L, sizeof(T)), s, a, L.carve);
+}
+
 // r_in / isq (fine level only): form b = r * isq in the first pass (the
 // float32 V-cycle's entry); b is then written, not read
 template <typename T>
@@ -1958,14 +2149,13 @@ void first_impl(const DevLevel& L, const T* b, T* x, T* bc_zero, int nc, cudaStr
             a.dv = A.dinv;
             a.b = b;
             a.x = x;
-            use_compact(L, A, a);
             if (L.split) {
+                use_compact(L, A, a);
                 a.out = level_s<T>(L);
                 vlaunch<FineSplitPassBody<T, kPartLower>>(fine_blocks(c1, c2), kFineBlock,
                                                           fine_smem(L, sizeof(T)), s, a, L.carve);
             } else {
-                vlaunch<FinePassBody<T>>(fine_blocks(c1, c2), kFineBlock, fine_smem(L, sizeof(T)), s, a,
-                                         L.carve);
+                fine_pass<T>(L, A, a, s);
             }
         }
         return;
@@ -2032,9 +2222,7 @@ void pass_impl(const DevLevel& L, int col, int jmax, RowPart part, const T* b, T
     if (L.lpr == kFine) {
         a.z = z_out;
         a.isq = isq;
-        use_compact(L, A, a);
-        vlaunch<FinePassBody<T>>(fine_blocks(r0, r1), kFineBlock, fine_smem(L, sizeof(T)), s, a,
-                                 L.carve);
+        fine_pass<T>(L, A, a, s);
         return;
     }
     if (z_out) throw Error{AMG_EINVAL, "the fused float32 exit needs the fine-level kernels"};
@@ -2059,6 +2247,12 @@ void residual_restrict_impl(const DevLevel& L, const T* b, const T* x, T* r, T* 
             a.idx = L.agg;
             a.t = A.t;
             a.out = bc;
+            if (wide_level(L)) {
+                const int grid = fine_blocks(c1, L.n);
+                if (L.width == 4) vlaunch<WideResRestrictBody<T, SC, 4>>(grid, kFineBlock, 0, s, a);
+                else vlaunch<WideResRestrictBody<T, SC, 6>>(grid, kFineBlock, 0, s, a);
+                return;
+            }
             use_compact(L, A, a);
             vlaunch<FineResRestrictBody<T, SC>>(fine_blocks(c1, L.n), kFineBlock,
                                                 fine_smem(L, sizeof(T)), s, a, L.carve);
@@ -2294,15 +2488,15 @@ void launch_from_scaled32(int n, const float* zhat, const double* isq, double* z
 
 void launch_cg_residual(const DevLevel& L, const double* b, const double* x, double* r,
                         CgWork& w, int mode, double* out, cudaStream_t s) {
-    launch_kernel(k_cg_residual, reduction_blocks(L.n), kBlock, 0, s, L.n, L.sw, L.rlen, L.scol, L.sval,
-                                                           L.diag, b, x, r, w.partials,
-                                                           w.counters, w.sc, out, mode);
+    AMG_WIDTH_DISPATCH(L.width, (launch_kernel(k_cg_residual<W>, row_loop_blocks(L), kBlock, 0, s, L.n, L.sw,
+                                               L.rlen, L.scol, L.sval, L.diag, b, x, r, w.partials,
+                                               w.counters, w.sc, out, mode)));
 }
 
 void launch_cg_spmv_pq(const DevLevel& L, const double* p, double* q, CgWork& w, cudaStream_t s) {
-    launch_kernel(k_cg_spmv_pq, reduction_blocks(L.n), kBlock, 0, s, L.n, L.sw, L.rlen, L.scol, L.sval,
-                                                          L.diag, p, q, w.partials,
-                                                          w.counters + 1, w.sc);
+    AMG_WIDTH_DISPATCH(L.width, (launch_kernel(k_cg_spmv_pq<W>, row_loop_blocks(L), kBlock, 0, s, L.n, L.sw,
+                                               L.rlen, L.scol, L.sval, L.diag, p, q, w.partials,
+                                               w.counters + 1, w.sc)));
 }
 
 void wait_selftest(long long limit, cudaStream_t s, int32_t* status, double* elapsed_ms) {
@@ -2349,8 +2543,9 @@ void launch_cg_p(int n, const double* z, double* p, double* zold, const CgWork& 
 
 void launch_bi_start(const DevLevel& L, const double* b, const double* x, double* r, double* rt,
                      CgWork& wk, BiScalars* bs, cudaStream_t s) {
-    launch_kernel(k_bi_start, reduction_blocks(L.n), kBlock, 0, s, L.n, L.sw, L.rlen, L.scol,
-                  L.sval, L.diag, b, x, r, rt, wk.partials, wk.partials2, wk.counters + 4, bs);
+    AMG_WIDTH_DISPATCH(L.width, (launch_kernel(k_bi_start<W>, row_loop_blocks(L), kBlock, 0, s, L.n, L.sw,
+                                               L.rlen, L.scol, L.sval, L.diag, b, x, r, rt, wk.partials,
+                                               wk.partials2, wk.counters + 4, bs)));
 }
 
 void launch_bi_direction(int n, const double* r, const double* v, double* p, const BiScalars* bs,
@@ -2360,9 +2555,10 @@ void launch_bi_direction(int n, const double* r, const double* v, double* p, con
 
 void launch_bi_spmv(const DevLevel& L, const double* x, double* y, const double* w, bool second,
                     CgWork& wk, BiScalars* bs, cudaStream_t s) {
-    launch_kernel(k_bi_spmv, reduction_blocks(L.n), kBlock, 0, s, L.n, L.sw, L.rlen, L.scol,
-                  L.sval, L.diag, x, y, w, wk.partials, wk.partials2, wk.counters + (second ? 6 : 5),
-                  bs, second ? (int)kBiW : (int)kBiRtv);
+    AMG_WIDTH_DISPATCH(L.width, (launch_kernel(k_bi_spmv<W>, row_loop_blocks(L), kBlock, 0, s, L.n, L.sw,
+                                               L.rlen, L.scol, L.sval, L.diag, x, y, w, wk.partials,
+                                               wk.partials2, wk.counters + (second ? 6 : 5), bs,
+                                               second ? (int)kBiW : (int)kBiRtv)));
 }
 
 void launch_bi_half(int n, const double* r, const double* v, double* sv, CgWork& wk,
