@@ -306,6 +306,12 @@ constexpr int64_t kMaxStageBytes = 96 * 1024;
 inline int64_t stage_bytes(const DevLevel& L, size_t value_bytes) {
     return L.stage_cap * (int64_t)(sizeof(int32_t) + value_bytes);
 }
+// the slice widths with kernels of their own, the 5-point and 7-point stencils:
+// their rows are read into registers, not staged (kernels.cu: WideRow)
+inline bool wide_rows(int width) { return width == 4 || width == 6; }
+inline bool wide_level(const DevLevel& L) { return !L.split && !L.soff && wide_rows(L.width); }
+// whether lanes per row 0 stages the level's slices in shared memory
+inline bool uses_shared_memory(const DevLevel& L) { return !wide_level(L); }
 inline bool staged_fits(const DevLevel& L) { return stage_bytes(L, sizeof(double)) <= kMaxStageBytes; }
 
 // Launch profiler: events around launches, grouped by kernel class.
@@ -612,6 +618,54 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
 // the map on the host.
 AggResult aggregate_tiles_device(const DevCsr& A, const amg_params& p, cudaStream_t s);
 
+// The coarsest matrix in the order of a dissection (rows: the parts, then the
+// separator; see host_setup.h), eliminated part by part:
+//   B = A_II^-1 (block diagonal), W = A_SI B, S = (A_SS - W A_IS)^-1;
+//   y = B b_I and t = b_S - W b_I;  x_S = S t;  x_I = y - W^T x_S.
+// The products read about a quarter of the entries of the whole inverse.
+struct DissDesc {
+    int32_t nI, ns, nblk, longest;    // rows of the parts, of the separator; blocks of 16 rows of
+                                      // a part; rows of the longest part
+    int32_t most_adj, pad;            // separator rows next to one part, at most
+    const int32_t* segp;              // [ns+1] a separator row's segments of W ...
+    const int32_t* seg;               // ... first column, length, place in W (3 per segment)
+    const double* W;
+    const double* S;                  // [ns][ns]
+    const int32_t* blk;               // 16 rows of a part: the part's first row, length, place in B,
+                                      // first row of the block; the part's separator rows: place
+                                      // in adj, number, place in WT (kDissBlk per block)
+    const int32_t* adj;               // separator rows next to each part, ascending
+    const double* B;                  // dense inverses of the parts
+    const double* WT;                 // W^T, row by row of each part over its separator rows
+    double* y;                        // [nI]
+    double* t;                        // [ns]
+    double* xs;                       // [ns]
+};
+constexpr int kDissRows = 16;         // rows of a part per block
+constexpr int kDissBlk = 8;
+
+struct Dissected {
+    bool on = false;
+    const DissDesc* desc[2] = {nullptr, nullptr};   // device: float64, and scaled by S = diag(sqrt(A_ii))
+    DissDesc host[2];
+    int64_t entries = 0;              // stored entries the products read
+    // for the scaled copy: segments' separator rows (device), parts, array sizes
+    const int32_t* grow = nullptr;
+    std::vector<int32_t> part_ptr, adj_ptr;
+    int64_t nW = 0, nB = 0;
+    int n_seg = 0;
+};
+
+// Builds the dissected coarsest solve in out (float64 values); false when a
+// pivot is not positive.  A is in its original order.
+bool dissect_device(const HostCsr& A, const Dissection& P, DevArena& arena, Dissected& out,
+                    cudaStream_t s);
+// its copy for the level scaled by S = diag(sqrt(diag)) (diag in the order of the dissection)
+void dissect_scaled(Dissected& d, const double* diag, DevArena& arena, cudaStream_t s);
+// x = A^-1 b
+void launch_dissected(const Dissected& d, const double* b, double* x, cudaStream_t s);
+void launch_dissected32(const Dissected& d, const float* b, float* x, cudaStream_t s);
+
 // Dense inverse of the (original-order) coarsest matrix through a Cholesky
 // factorisation of its lower triangle; returns false when a pivot is not
 // positive.
@@ -682,6 +736,7 @@ struct amg_ctx {
     int32_t nL = 0;                   // coarsest size
     double* Ainv = nullptr;           // [nL x nL] inverse of the coarsest matrix
     double* Ainv_s = nullptr;         // [nL x nL] inverse of the scaled coarsest matrix
+    amg::Dissected diss;              // instead of the dense inverses, on larger coarsest levels
     float* Ainv_s32 = nullptr;        // its float32 copy, rows of ld32 floats (coarsest_fp32 only)
     int ld32 = 0;                     // nL rounded up to a multiple of 4
     double* isq0 = nullptr;           // [n] 1 / sqrt(A_ii) of level 0 (FP32 entry/exit)

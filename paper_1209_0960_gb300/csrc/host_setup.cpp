@@ -807,4 +807,91 @@ int32_t smoother_colouring(const HostCsr& A, std::vector<int32_t>& colour) {
     return nc;
 }
 
+Dissection dissect(const HostCsr& A, int depth) {
+    const int32_t n = A.n;
+    std::vector<std::vector<int32_t>> parts(1);
+    parts[0].resize(n);
+    for (int32_t i = 0; i < n; ++i) parts[0][i] = i;
+    std::vector<int32_t> sep, in(n, 0), du(n), dw(n), order, pos(n);
+    int32_t mark = 0;
+    // breadth-first order of the marked rows from src, distances into d (-1: not reached)
+    auto bfs = [&](int32_t src, const std::vector<int32_t>& V, std::vector<int32_t>& d) {
+        for (int32_t v : V) d[v] = -1;
+        order.clear();
+        order.push_back(src);
+        d[src] = 0;
+        for (size_t q = 0; q < order.size(); ++q) {
+            const int32_t v = order[q];
+            for (int32_t k = A.rp[v]; k < A.rp[v + 1]; ++k) {
+                const int32_t w = A.ci[k];
+                if (in[w] == mark && d[w] < 0) {
+                    d[w] = d[v] + 1;
+                    order.push_back(w);
+                }
+            }
+        }
+    };
+    for (int level = 0; level < depth; ++level) {
+        std::vector<std::vector<int32_t>> next;
+        for (std::vector<int32_t>& V : parts) {
+            if (V.size() < 2) {
+                next.push_back(std::move(V));
+                continue;
+            }
+            ++mark;
+            for (int32_t v : V) in[v] = mark;
+            bfs(V[0], V, du);
+            if (order.size() < V.size()) {   // not connected: no separator needed
+                std::vector<int32_t> a = order, b;
+                for (int32_t v : V)
+                    if (du[v] < 0) b.push_back(v);
+                next.push_back(std::move(a));
+                next.push_back(std::move(b));
+                continue;
+            }
+            for (int rep = 0; rep < 2; ++rep) bfs(order.back(), V, du);
+            bfs(order.back(), V, dw);
+            std::vector<int32_t> o = V;
+            std::sort(o.begin(), o.end(), [&](int32_t a, int32_t b) {
+                const int32_t ka = du[a] - dw[a], kb = du[b] - dw[b];
+                return ka != kb ? ka < kb : a < b;
+            });
+            const int32_t m = (int32_t)o.size();
+            for (int32_t k = 0; k < m; ++k) pos[o[k]] = k;
+            // edge[k]: rows before k with a neighbour at or behind k
+            std::vector<int32_t> last(m), edge(m + 1, 0);
+            for (int32_t q = 0; q < m; ++q) {
+                int32_t far = q;
+                for (int32_t k = A.rp[o[q]]; k < A.rp[o[q] + 1]; ++k)
+                    if (in[A.ci[k]] == mark) far = std::max(far, pos[A.ci[k]]);
+                last[q] = far;
+                if (far > q) {
+                    ++edge[q + 1];
+                    if (far + 1 <= m) --edge[far + 1];
+                }
+            }
+            for (int32_t k = 1; k <= m; ++k) edge[k] += edge[k - 1];
+            int32_t cut = std::max(1, (int32_t)(0.4 * m));
+            for (int32_t k = cut; k <= (int32_t)(0.6 * m) && k < m; ++k)
+                if (edge[k] < edge[cut]) cut = k;
+            std::vector<int32_t> a, b(o.begin() + cut, o.end());
+            for (int32_t q = 0; q < cut; ++q) (last[q] >= cut ? sep : a).push_back(o[q]);
+            next.push_back(std::move(a));
+            next.push_back(std::move(b));
+        }
+        parts = std::move(next);
+    }
+    Dissection D;
+    D.ptr.push_back(0);
+    for (std::vector<int32_t>& V : parts) {
+        if (V.empty()) continue;
+        std::sort(V.begin(), V.end());
+        D.order.insert(D.order.end(), V.begin(), V.end());
+        D.ptr.push_back((int32_t)D.order.size());
+    }
+    std::sort(sep.begin(), sep.end());
+    D.order.insert(D.order.end(), sep.begin(), sep.end());
+    return D;
+}
+
 }  // namespace amg

@@ -59,4 +59,18 @@ int32_t dsatur_colouring(const HostCsr& A, std::vector<int32_t>& colour);
 // ascending-order greedy, else the greedy one.
 int32_t smoother_colouring(const HostCsr& A, std::vector<int32_t>& colour);
 
+// A nested dissection of the graph of A into np parts without entries between
+// them and a separator: order lists the rows part by part, the separator last;
+// part k is order[ptr[k], ptr[k+1]), the separator order[ptr[np], n).
+struct Dissection {
+    std::vector<int32_t> order, ptr;
+    int parts() const { return (int)ptr.size() - 1; }
+};
+
+// Splits the graph `depth` times in halves by vertex separators: the rows of a
+// half in the order of d(u) - d(w), the breadth-first distances from two far
+// ends u and w, cut where the fewest rows before the cut have a neighbour
+// behind it (between 40 and 60 % of the half); those rows join the separator.
+Dissection dissect(const HostCsr& A, int depth);
+
 }  // namespace amg

@@ -1460,6 +1460,139 @@ struct GemvF32Body {
     }
 };
 
+// The dissected coarsest solve (DissDesc) in three launches.  The float64 pipe
+// sets the time of a coarsest solve: the whole inverse of 4,645 rows is 21.6M
+// multiply-adds, about 37 us at two a clock per SM, the products here about a
+// quarter of that.  128^3 (4,645 rows), V-cycle: float64 422 -> 380-390 us, mixed
+// 324 -> 297 us; and 90 ms of setup less.  (With x_I = B (b_I - A_IS x_S), a
+// quarter fewer entries, every block formed its part's right-hand side again:
+// 35 us for that launch alone against 13.)  Sums run over 32 lanes of long rows, and over 8 lanes
+// of the parts' rows, whose sums across lanes would otherwise cost a third of
+// their multiply-adds.  Arguments: dv = descriptor, b, x.
+
+// this lane's share (elements lane, lane + G, ...) of m . v, U loads in flight; a
+// last partial batch is predicated, not looped: one by one its loads would each
+// cost a round trip
+template <int G, int U>
+__device__ __forceinline__ double lane_dot(const double* __restrict__ m, const double* v, int len,
+                                           int lane, double s) {
+    for (int k0 = lane; k0 < len; k0 += G * U) {
+        double a[U], c[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool in = k0 + u * G < len;
+            a[u] = in ? m[k0 + u * G] : 0.0;
+            c[u] = in ? v[k0 + u * G] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k0 - lane + u * G < len) s = fmad(a[u], c[u], s);   // the same for all lanes
+    }
+    return s;
+}
+
+// y = B b_I (blocks [0, nblk): 16 rows of a part each, two rows a warp) and
+// t = b_S - W b_I (one warp per separator row); the block first copies b into
+// shared memory (as float64), a part's block its part only.  128 threads a
+// block.
+constexpr int kDissThreads = 128;
+template <typename TB>
+struct DissFirstBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        constexpr int G = kDissThreads / kDissRows;
+        const DissDesc& D = *static_cast<const DissDesc*>(a.dv);
+        const TB* b = static_cast<const TB*>(a.b);
+        extern __shared__ double sbuf[];
+        trigger_early(a);
+        const int nI = D.nI, ns = D.ns, nblk = D.nblk, tid = (int)threadIdx.x;
+        const bool part = bid < nblk;
+        const int32_t* q = D.blk + kDissBlk * (part ? bid : 0);
+        const int p0 = part ? q[0] : 0, len = part ? q[1] : nI;
+        const double* B = D.B + (size_t)q[2];
+        const int r = (part ? q[3] : 0) + tid / G;
+        const int row = (bid - nblk) * (kDissThreads / 32) + (tid >> 5);
+        const int32_t* seg = D.seg;
+        const int g0 = !part && row < ns ? D.segp[row] : 0, g1 = !part && row < ns ? D.segp[row + 1] : 0;
+        const double* W = D.W;
+        double* y = D.y;
+        double* t = D.t;
+        wait_and_trigger(a);
+#pragma unroll 8
+        for (int k = tid; k < len; k += kDissThreads) sbuf[k] = (double)b[p0 + k];
+        __syncthreads();
+        const double* sb = sbuf;   // b_I from row p0 on
+        if (part) {
+            const int lane = tid % G;
+            const double s =
+                group_sum<G>(lane_dot<G, 16>(B + (size_t)min(r, len - 1) * len, sb, len, lane, 0.0));
+            if (r < len && lane == 0) y[p0 + r] = s;
+        } else if (row < ns) {
+            const int lane = tid & 31;
+            double s = 0.0;
+            for (int g = g0; g < g1; ++g)
+                s = lane_dot<32, 16>(W + (size_t)seg[3 * g + 2], sb + seg[3 * g], seg[3 * g + 1], lane, s);
+            s = group_sum<32>(s);
+            if (lane == 0) t[row] = (double)b[nI + row] - s;
+        }
+    }
+};
+
+// x_S = S t, one warp per row
+template <typename TB>
+struct DissSepBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        const DissDesc& D = *static_cast<const DissDesc*>(a.dv);
+        TB* x = static_cast<TB*>(a.x);
+        trigger_early(a);
+        const int lane = threadIdx.x & 31;
+        const int row = (int)((bid * (int64_t)blockDim.x + threadIdx.x) >> 5);
+        const int ns = D.ns, nI = D.nI;
+        const double* m = D.S + (size_t)min(row, ns - 1) * ns;
+        const double* t = D.t;
+        double* xs = D.xs;
+        wait_and_trigger(a);
+        if (row >= ns) return;
+        const double s = group_sum<32>(lane_dot<32, 16>(m, t, ns, lane, 0.0));
+        if (lane == 0) {
+            xs[row] = s;
+            x[nI + row] = (TB)s;
+        }
+    }
+};
+
+// x_I = y - W^T x_S: a block takes 16 rows of a part, gathers the part's
+// separator values into shared memory and sums each row over 8 lanes
+template <typename TB>
+struct DissPartBody {
+    static __device__ __forceinline__ void run(int bid, int, const VArgs& a) {
+        constexpr int G = kDissThreads / kDissRows;
+        const DissDesc& D = *static_cast<const DissDesc*>(a.dv);
+        TB* x = static_cast<TB*>(a.x);
+        extern __shared__ double sbuf[];
+        trigger_early(a);
+        const int tid = (int)threadIdx.x;
+        const int32_t* q = D.blk + kDissBlk * bid;
+        const int p0 = q[0], len = q[1], na = q[5], lane = tid % G, r = q[3] + tid / G;
+        const int32_t* adj = D.adj + q[4];
+        const double* m = D.WT + (size_t)q[6] + (size_t)min(r, len - 1) * na;
+        const double* xs = D.xs;
+        const double* y = D.y;
+        constexpr int kAt = 8;
+        int j[kAt];
+#pragma unroll
+        for (int u = 0; u < kAt; ++u) j[u] = tid + u * kDissThreads < na ? adj[tid + u * kDissThreads] : -1;
+        wait_and_trigger(a);
+#pragma unroll
+        for (int u = 0; u < kAt; ++u)
+            if (j[u] >= 0) sbuf[tid + u * kDissThreads] = xs[j[u]];
+        for (int k = tid + kAt * kDissThreads; k < na; k += kDissThreads) sbuf[k] = xs[adj[k]];
+        const double yr = r < len ? y[p0 + r] : 0.0;
+        __syncthreads();
+        const double s = group_sum<G>(lane_dot<G, 16>(m, sbuf, na, lane, 0.0));
+        if (r < len && lane == 0) x[p0 + r] = (TB)(yr - s);
+    }
+};
+
 __global__ void k_gather(int n, const int32_t* __restrict__ idx, const double* x, double* y) {
     pdl_launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1972,14 +2105,12 @@ inline int launch_lpr(const DevLevel& L, int rows) {
     return rows >= L.wide_rows ? L.lpr_wide : L.lpr;
 }
 
-// the slice widths with kernels of their own: the 5-point and 7-point stencils
 #define AMG_WIDTH_DISPATCH(width, CALL)              \
     switch (width) {                                 \
         case 4: { constexpr int W = 4; CALL; } break;  \
         case 6: { constexpr int W = 6; CALL; } break;  \
         default: { constexpr int W = 0; CALL; } break; \
     }
-inline bool wide_rows(int width) { return width == 4 || width == 6; }
 // grid of a CG kernel over rows: four blocks per SM with RowLoop<W > 0>, else eight
 inline int row_loop_blocks(const DevLevel& L) {
     const int b = reduction_blocks(L.n);
@@ -2104,9 +2235,6 @@ void use_compact(const DevLevel& L, const LevelArrays<T>& A, VArgs& a) {
     a.scol = L.ccol;
     a.sval = A.cval;
 }
-
-// levels of the staged kernels (lanes per row 0) that WideRow covers
-inline bool wide_level(const DevLevel& L) { return !L.split && !L.soff && wide_rows(L.width); }
 
 // one colour pass of a level that is not split, by the one-row-per-thread kernels
 template <typename T>
@@ -2434,6 +2562,26 @@ void launch_dense_gemv(int n, const double* M, const double* b, double* x, cudaS
 
 void launch_dense_gemv32(int n, const double* M, const float* b, float* x, cudaStream_t s) {
     dense_gemv_impl<float>(n, M, b, x, s);
+}
+
+template <typename TB>
+void dissected_impl(const DissDesc& D, const DissDesc* dev, const TB* b, TB* x, cudaStream_t s) {
+    VArgs a;
+    a.dv = dev;
+    a.b = b;
+    a.x = x;
+    const size_t smem = sizeof(double) * (size_t)(D.ns > 0 ? D.nI : D.longest);
+    vlaunch<DissFirstBody<TB>>(D.nblk + (D.ns + kDissThreads / 32 - 1) / (kDissThreads / 32), kDissThreads,
+                               smem, s, a);
+    if (D.ns > 0) vlaunch<DissSepBody<TB>>((D.ns + kDissThreads / 32 - 1) / (kDissThreads / 32), kDissThreads, 0, s, a);
+    vlaunch<DissPartBody<TB>>(D.nblk, kDissThreads, sizeof(double) * (size_t)std::max(1, D.most_adj), s, a);
+}
+
+void launch_dissected(const Dissected& d, const double* b, double* x, cudaStream_t s) {
+    dissected_impl<double>(d.host[0], d.desc[0], b, x, s);
+}
+void launch_dissected32(const Dissected& d, const float* b, float* x, cudaStream_t s) {
+    dissected_impl<float>(d.host[1], d.desc[1], b, x, s);
 }
 
 void launch_vrecords(const VRec* const* recs, int n, cudaStream_t s) {

@@ -628,18 +628,15 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
 }
 
-bool dense_inverse_device(const DevCsr& A, double* Minv, cudaStream_t s) {
-    const int n = A.n;
+// Minv = W^-1 for the dense matrix whose lower triangle is W (overwritten)
+static bool invert_dense(int n, double* W, double* Minv, cudaStream_t s) {
     const int np = (n + kPanel - 1) / kPanel;
     DevArena tmp(s);
-    double* W = tmp.alloc<double>((size_t)n * n);
     double* Y = tmp.alloc<double>((size_t)n * n);
     double* D = tmp.alloc<double>((size_t)np * kPanel * kPanel);
     int* err = tmp.alloc<int>(1);
-    AMG_CUDA_TRY(cudaMemsetAsync(W, 0, sizeof(double) * (size_t)n * n, s));
     AMG_CUDA_TRY(cudaMemsetAsync(Y, 0, sizeof(double) * (size_t)n * n, s));
     AMG_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
-    k_dense_from_csr<<<blocks_for(n), kBlock, 0, s>>>(n, A.rp, A.ci, A.va, W);
     // Cholesky, right-looking by 32-column panels
     for (int p = 0; p < np; ++p) {
         const int k0 = p * kPanel, m = std::min(kPanel, n - k0), r0 = k0 + m;
@@ -667,6 +664,298 @@ bool dense_inverse_device(const DevCsr& A, double* Minv, cudaStream_t s) {
     AMG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
     return herr == 0;
+}
+
+bool dense_inverse_device(const DevCsr& A, double* Minv, cudaStream_t s) {
+    const int n = A.n;
+    DevArena tmp(s);
+    double* W = tmp.alloc<double>((size_t)n * n);
+    AMG_CUDA_TRY(cudaMemsetAsync(W, 0, sizeof(double) * (size_t)n * n, s));
+    k_dense_from_csr<<<blocks_for(n), kBlock, 0, s>>>(n, A.rp, A.ci, A.va, W);
+    return invert_dense(n, W, Minv, s);
+}
+
+// ---------------------------------------------------------------------------
+// the dissected coarsest solve (see DissDesc)
+// ---------------------------------------------------------------------------
+namespace {
+
+// W rows: segment g of a separator row is sum_l a_il B_k[l][.] over the row's
+// entries l in part k.  One block per segment.
+__global__ void k_diss_w(const int32_t* __restrict__ gseg, const int32_t* __restrict__ grow,
+                         const int32_t* __restrict__ spp, const int32_t* __restrict__ spc,
+                         const double* __restrict__ spv, const int64_t* __restrict__ boff,
+                         const double* __restrict__ B, double* __restrict__ W) {
+    const int g = (int)blockIdx.x;
+    const int p0 = gseg[3 * g], len = gseg[3 * g + 1], at = gseg[3 * g + 2], i = grow[g];
+    const double* Bk = B + boff[g];
+    for (int j = threadIdx.x; j < len; j += blockDim.x) {
+        double s = 0.0;
+        for (int k = spp[i]; k < spp[i + 1]; ++k) {
+            const int l = spc[k] - p0;
+            if (l >= 0 && l < len) s = fma(spv[k], Bk[(size_t)l * len + j], s);
+        }
+        W[(size_t)at + j] = s;
+    }
+}
+
+// Schur complement, lower triangle: S_ij = A_ij - sum_l W_il a_jl over the
+// interior entries l of row j
+__global__ void k_diss_schur(int ns, const int32_t* __restrict__ segp, const int32_t* __restrict__ seg,
+                             const double* __restrict__ W, const int32_t* __restrict__ spp,
+                             const int32_t* __restrict__ spc, const double* __restrict__ spv,
+                             double* __restrict__ S) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int i = (int)(t / ns), j = (int)(t % ns);
+    if (i >= ns || j > i) return;
+    double s = 0.0;
+    for (int k = spp[j]; k < spp[j + 1]; ++k) {
+        const int l = spc[k];
+        for (int g = segp[i]; g < segp[i + 1]; ++g) {
+            const int q = l - seg[3 * g];
+            if (q >= 0 && q < seg[3 * g + 1]) s = fma(W[(size_t)seg[3 * g + 2] + q], spv[k], s);
+        }
+    }
+    S[(size_t)i * ns + j] -= s;
+}
+
+__global__ void k_diss_fill(int m, const int32_t* __restrict__ at_r, const int32_t* __restrict__ at_c,
+                            const double* __restrict__ v, int ns, double* __restrict__ S) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < m) S[(size_t)at_r[k] * ns + at_c[k]] = v[k];
+}
+
+// scaled copies: entry (r, c) times sqrt(d_r)^pr sqrt(d_c)^pc
+__global__ void k_diss_scale_dense(int64_t count, int r0, int len, const double* __restrict__ diag,
+                                   const double* __restrict__ in, double* __restrict__ out) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= count) return;
+    out[t] = sqrt(diag[r0 + t / len]) * in[t] * sqrt(diag[r0 + t % len]);
+}
+__global__ void k_diss_scale_w(int nI, const int32_t* __restrict__ gseg, const int32_t* __restrict__ grow,
+                               const double* __restrict__ diag, const double* __restrict__ in,
+                               double* __restrict__ out) {
+    const int g = (int)blockIdx.x;
+    const int p0 = gseg[3 * g], len = gseg[3 * g + 1];
+    const size_t at = (size_t)gseg[3 * g + 2];
+    const double si = sqrt(diag[nI + grow[g]]);
+    for (int j = threadIdx.x; j < len; j += blockDim.x) out[at + j] = in[at + j] * sqrt(diag[p0 + j]) / si;
+}
+__global__ void k_diss_scale_wt(int64_t count, int p0, int m, int nI, const int32_t* __restrict__ adj,
+                                const double* __restrict__ diag, const double* __restrict__ in,
+                                double* __restrict__ out) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= count) return;
+    out[t] = in[t] * sqrt(diag[p0 + t / m]) / sqrt(diag[nI + adj[t % m]]);
+}
+
+// W^T of one part: row l over the part's separator rows (j-th: its segment starts at place[j])
+__global__ void k_diss_wt(int len, int m, const int32_t* __restrict__ place, const double* __restrict__ W,
+                          double* __restrict__ WT) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= (int64_t)len * m) return;
+    const int l = (int)(t / m), j = (int)(t % m);
+    WT[t] = W[(size_t)place[j] + l];
+}
+
+template <typename T>
+T* to_device(DevArena& arena, const std::vector<T>& v, cudaStream_t s) {
+    T* d = arena.alloc<T>(v.size());
+    if (!v.empty())
+        AMG_CUDA_TRY(cudaMemcpyAsync(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s));
+    return d;
+}
+
+}  // namespace
+
+bool dissect_device(const HostCsr& A, const Dissection& P, DevArena& arena, Dissected& out,
+                    cudaStream_t s) {
+    const int np = P.parts();
+    const int32_t n = A.n, nI = P.ptr[np], ns = n - nI;
+    DevArena tmp(s);
+    std::vector<int32_t> pos(n), part(n, -1);
+    for (int32_t k = 0; k < n; ++k) pos[P.order[k]] = k;
+    for (int k = 0; k < np; ++k)
+        for (int32_t q = P.ptr[k]; q < P.ptr[k + 1]; ++q) part[P.order[q]] = k;
+    // dense inverses of the parts
+    std::vector<int64_t> b0(np + 1, 0);
+    for (int k = 0; k < np; ++k) {
+        const int64_t m = P.ptr[k + 1] - P.ptr[k];
+        b0[k + 1] = b0[k] + m * m;
+    }
+    double* B = arena.alloc<double>((size_t)b0[np]);
+    int32_t longest = 1;
+    for (int k = 0; k < np; ++k) {
+        const int32_t p0 = P.ptr[k], m = P.ptr[k + 1] - p0;
+        longest = std::max(longest, m);
+        HostCsr sub;
+        sub.n = m;
+        sub.rp.assign(m + 1, 0);
+        for (int32_t q = 0; q < m; ++q) {
+            const int32_t i = P.order[p0 + q];
+            for (int32_t e = A.rp[i]; e < A.rp[i + 1]; ++e)
+                if (part[A.ci[e]] == k) {
+                    sub.ci.push_back(pos[A.ci[e]] - p0);
+                    sub.va.push_back(A.va[e]);
+                }
+            sub.rp[q + 1] = (int32_t)sub.ci.size();
+        }
+        DevArena sm(s);
+        DevCsr D;
+        D.n = m;
+        D.nnz = sub.nnz();
+        D.rp = to_device(sm, sub.rp, s);
+        D.ci = to_device(sm, sub.ci, s);
+        D.va = to_device(sm, sub.va, s);
+        if (!dense_inverse_device(D, B + b0[k], s)) return false;   // (waits for the stream)
+    }
+    // separator rows: interior entries, segments of W, A_SS
+    std::vector<int32_t> spp(1, 0), spc, segp(1, 0), seg, grow, ssr, ssc;
+    std::vector<int64_t> gb;
+    std::vector<double> spv, ssv;
+    std::vector<std::vector<int32_t>> adj(np), place(np);   // a part's separator rows, their W segments
+    int64_t nW = 0;
+    std::vector<char> has(np);
+    for (int32_t q = 0; q < ns; ++q) {
+        const int32_t i = P.order[nI + q];
+        std::fill(has.begin(), has.end(), 0);
+        for (int32_t e = A.rp[i]; e < A.rp[i + 1]; ++e) {
+            const int32_t j = A.ci[e];
+            if (part[j] >= 0) {
+                spc.push_back(pos[j]);
+                spv.push_back(A.va[e]);
+                has[part[j]] = 1;
+            } else if (pos[j] - nI <= q) {
+                ssr.push_back(q);
+                ssc.push_back(pos[j] - nI);
+                ssv.push_back(A.va[e]);
+            }
+        }
+        spp.push_back((int32_t)spc.size());
+        for (int k = 0; k < np; ++k)
+            if (has[k]) {
+                const int32_t m = P.ptr[k + 1] - P.ptr[k];
+                seg.insert(seg.end(), {P.ptr[k], m, (int32_t)nW});
+                grow.push_back(q);
+                gb.push_back(b0[k]);
+                adj[k].push_back(q);
+                place[k].push_back((int32_t)nW);
+                nW += m;
+            }
+        segp.push_back((int32_t)grow.size());
+    }
+    // blocks of kDissRows rows
+    std::vector<int32_t> blk, adj_all, adj_ptr(1, 0);
+    std::vector<int64_t> wt0(np, 0);
+    int32_t most_adj = 0;
+    {
+        int64_t at = 0;
+        for (int k = 0; k < np; ++k) {
+            const int32_t p0 = P.ptr[k], m = P.ptr[k + 1] - p0, na = (int32_t)adj[k].size();
+            wt0[k] = at;
+            for (int32_t r = 0; r < m; r += kDissRows)
+                blk.insert(blk.end(), {p0, m, (int32_t)b0[k], r, (int32_t)adj_all.size(), na, (int32_t)at, 0});
+            adj_all.insert(adj_all.end(), adj[k].begin(), adj[k].end());
+            adj_ptr.push_back((int32_t)adj_all.size());
+            most_adj = std::max(most_adj, na);
+            at += (int64_t)m * na;
+        }
+    }
+    const int ng = (int)grow.size();
+    int32_t* d_seg = to_device(arena, seg, s);
+    int32_t* d_segp = to_device(arena, segp, s);
+    int32_t* d_grow = to_device(arena, grow, s);
+    int32_t* d_spp = to_device(tmp, spp, s);
+    int32_t* d_spc = to_device(tmp, spc, s);
+    double* d_spv = to_device(tmp, spv, s);
+    int64_t* d_gb = to_device(tmp, gb, s);
+    double* W = arena.alloc<double>((size_t)nW);
+    double* WT = arena.alloc<double>((size_t)nW);
+    double* S = arena.alloc<double>((size_t)ns * ns);
+    if (ng > 0) {
+        k_diss_w<<<ng, 128, 0, s>>>(d_seg, d_grow, d_spp, d_spc, d_spv, d_gb, B, W);
+        for (int k = 0; k < np; ++k) {
+            const int len = P.ptr[k + 1] - P.ptr[k], m = (int)adj[k].size();
+            if (m > 0)
+                k_diss_wt<<<blocks_for((int64_t)len * m), kBlock, 0, s>>>(len, m, to_device(tmp, place[k], s),
+                                                                          W, WT + wt0[k]);
+        }
+        AMG_CUDA_TRY(cudaGetLastError());
+    }
+    bool ok = true;
+    if (ns > 0) {
+        double* M = tmp.alloc<double>((size_t)ns * ns);
+        AMG_CUDA_TRY(cudaMemsetAsync(M, 0, sizeof(double) * (size_t)ns * ns, s));
+        k_diss_fill<<<blocks_for((int64_t)ssr.size()), kBlock, 0, s>>>(
+            (int)ssr.size(), to_device(tmp, ssr, s), to_device(tmp, ssc, s), to_device(tmp, ssv, s), ns, M);
+        k_diss_schur<<<blocks_for((int64_t)ns * ns), kBlock, 0, s>>>(ns, d_segp, d_seg, W, d_spp, d_spc,
+                                                                     d_spv, M);
+        AMG_CUDA_TRY(cudaGetLastError());
+        ok = invert_dense(ns, M, S, s);
+    }
+    DissDesc& d = out.host[0];
+    d.nI = nI;
+    d.ns = ns;
+    d.nblk = (int32_t)(blk.size() / kDissBlk);
+    d.longest = longest;
+    d.most_adj = most_adj;
+    d.segp = d_segp;
+    d.seg = d_seg;
+    d.W = W;
+    d.S = S;
+    d.blk = to_device(arena, blk, s);
+    d.adj = to_device(arena, adj_all, s);
+    d.B = B;
+    d.WT = WT;
+    d.y = arena.alloc<double>(nI);
+    d.t = arena.alloc<double>(ns);
+    d.xs = arena.alloc<double>(ns);
+    DissDesc* dev = arena.alloc<DissDesc>(1);
+    AMG_CUDA_TRY(cudaMemcpyAsync(dev, &d, sizeof(DissDesc), cudaMemcpyHostToDevice, s));
+    out.desc[0] = dev;
+    out.grow = d_grow;
+    out.part_ptr = P.ptr;
+    out.nW = nW;
+    out.nB = b0[np];
+    out.n_seg = ng;
+    out.adj_ptr = adj_ptr;
+    out.entries = 2 * nW + b0[np] + (int64_t)ns * ns;
+    out.on = true;
+    AMG_CUDA_TRY(cudaStreamSynchronize(s));
+    return ok;
+}
+
+void dissect_scaled(Dissected& o, const double* diag, DevArena& arena, cudaStream_t s) {
+    DissDesc& d = o.host[1];
+    d = o.host[0];
+    double* W = arena.alloc<double>((size_t)o.nW);
+    double* S = arena.alloc<double>((size_t)d.ns * d.ns);
+    double* B = arena.alloc<double>((size_t)o.nB);
+    double* WT = arena.alloc<double>((size_t)o.nW);
+    if (o.n_seg > 0) k_diss_scale_w<<<o.n_seg, 128, 0, s>>>(d.nI, d.seg, o.grow, diag, d.W, W);
+    if (d.ns > 0) {
+        const int64_t m = (int64_t)d.ns * d.ns;
+        k_diss_scale_dense<<<blocks_for(m), kBlock, 0, s>>>(m, d.nI, d.ns, diag, d.S, S);
+    }
+    int64_t at = 0, wt = 0;
+    for (size_t k = 0; k + 1 < o.part_ptr.size(); ++k) {
+        const int len = o.part_ptr[k + 1] - o.part_ptr[k], na = o.adj_ptr[k + 1] - o.adj_ptr[k];
+        const int64_t m = (int64_t)len * len, w = (int64_t)len * na;
+        k_diss_scale_dense<<<blocks_for(m), kBlock, 0, s>>>(m, o.part_ptr[k], len, diag, d.B + at, B + at);
+        if (w > 0)
+            k_diss_scale_wt<<<blocks_for(w), kBlock, 0, s>>>(w, o.part_ptr[k], na, d.nI, d.adj + o.adj_ptr[k],
+                                                             diag, d.WT + wt, WT + wt);
+        at += m;
+        wt += w;
+    }
+    AMG_CUDA_TRY(cudaGetLastError());
+    d.W = W;
+    d.S = S;
+    d.B = B;
+    d.WT = WT;
+    DissDesc* dev = arena.alloc<DissDesc>(1);
+    AMG_CUDA_TRY(cudaMemcpyAsync(dev, &d, sizeof(DissDesc), cudaMemcpyHostToDevice, s));
+    o.desc[1] = dev;
 }
 
 __global__ void k_to_float_padded(int n, int ld, const double* __restrict__ in, float* __restrict__ out) {

@@ -158,12 +158,17 @@ double prolong_bytes(const DevLevel& L, int vb, bool scaled) {
     return m * (4 + 2.0 * vb + (scaled ? 4 : 0)) + (double)L.n_coarse * vb;
 }
 
-// modelled bytes of one V-cycle on a level, following the pass sequence of
-// vcycle64/vcycle32; the coarsest level reads its dense inverse once
-// mb: bytes per entry of the coarsest inverse as applied (8, or 4 for its
-// float32 copy in the float32 V-cycle)
-double level_vcycle_bytes(const DevLevel& L, bool coarsest, int vb, int mb = 8) {
-    if (coarsest) return (double)L.n * L.n * mb + 2.0 * L.n * vb;
+// the coarsest solve reads its dense inverse (in float32 with coarsest_fp32)
+// or the dissected one once
+double coarsest_bytes(const amg_ctx* c, int vb) {
+    const double n = c->nL;
+    if (c->diss.on) return 8.0 * (double)c->diss.entries + 2.0 * n * vb;
+    return n * n * (vb == 4 && c->p.coarsest_fp32 ? 4.0 : 8.0) + 2.0 * n * vb;
+}
+
+// modelled bytes of one V-cycle on a level above the coarsest, following the
+// pass sequence of vcycle64/vcycle32
+double level_vcycle_bytes(const DevLevel& L, int vb) {
     const bool scaled = vb == 4;
     const int C = L.ncolours;
     double t = first_bytes(L, vb);
@@ -192,8 +197,8 @@ void fill_info(amg_ctx* c) {
         li.max_agg_size = last ? 0 : h.agg.max_size;
         li.n_isolated = last ? 0 : h.agg.n_isolated;
         li.n_dirichlet = last ? 0 : h.agg.n_dirichlet;
-        li.vcycle_bytes_fp64 = level_vcycle_bytes(d, last, 8);
-        li.vcycle_bytes_fp32 = level_vcycle_bytes(d, last, 4, c->p.coarsest_fp32 ? 4 : 8);
+        li.vcycle_bytes_fp64 = last ? coarsest_bytes(c, 8) : level_vcycle_bytes(d, 8);
+        li.vcycle_bytes_fp32 = last ? coarsest_bytes(c, 4) : level_vcycle_bytes(d, 4);
         li.lanes_per_row = last ? 0 : d.lpr;
         li.threads_per_block = last ? 0 : d.block;
         li.sweep = (!last && d.sweep) ? 1 : 0;
@@ -306,9 +311,13 @@ inline void k_prolong(const DevLevel& L, const double* e, double* x, double w, c
 inline void k_prolong(const DevLevel& L, const float* e, float* x, double w, cudaStream_t s) { launch_prolong32(L, e, x, w, s); }
 inline void k_sweep(const DevLevel& L, const SweepPlan& P, const double* b, double* x, cudaStream_t s) { launch_sweep(L, P, b, x, s); }
 inline void k_sweep(const DevLevel& L, const SweepPlan& P, const float* b, float* x, cudaStream_t s) { launch_sweep32(L, P, b, x, s); }
-inline void k_coarsest(amg_ctx* c, const double* b, double* x) { launch_dense_gemv(c->nL, c->Ainv, b, x, c->stream); }
+inline void k_coarsest(amg_ctx* c, const double* b, double* x) {
+    if (c->diss.on) launch_dissected(c->diss, b, x, c->stream);
+    else launch_dense_gemv(c->nL, c->Ainv, b, x, c->stream);
+}
 inline void k_coarsest(amg_ctx* c, const float* b, float* x) {
-    if (c->Ainv_s32) launch_dense_gemv_f32(c->nL, c->ld32, c->Ainv_s32, b, x, c->stream);
+    if (c->diss.on) launch_dissected32(c->diss, b, x, c->stream);
+    else if (c->Ainv_s32) launch_dense_gemv_f32(c->nL, c->ld32, c->Ainv_s32, b, x, c->stream);
     else launch_dense_gemv32(c->nL, c->Ainv_s, b, x, c->stream);
 }
 
@@ -328,8 +337,7 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
     DevLevel& L = c->dl[l];
     cudaStream_t s = c->stream;
     if (l == nlev - 1) {
-        const double mb = (vb == 4 && c->Ainv_s32) ? 4.0 : 8.0;
-        ProfScope ps(c, kKCoarseSolve, (double)c->nL * c->nL * mb + 2.0 * vb * c->nL);
+        ProfScope ps(c, kKCoarseSolve, coarsest_bytes(c, vb));
         vkey(0, l, 0);
         k_coarsest(c, b, x);
         return;
@@ -352,8 +360,7 @@ void vcycle(amg_ctx* c, int l, const T* b, T* x) {
             }
         }
         if (t.one) {
-            const double mb = (vb == 4 && c->Ainv_s32) ? 4.0 : 8.0;
-            ProfScope ps(c, kKCoarseSolve, down + up + (double)c->nL * c->nL * mb + 2.0 * vb * c->nL);
+            ProfScope ps(c, kKCoarseSolve, down + up + coarsest_bytes(c, vb));
             vkey(0, l, 0);
             launch_tail(t.down, scaled, s);
             return;
@@ -516,8 +523,12 @@ void ensure_fp32(amg_ctx* c) {
         const double* cdiag = (l + 1 < nlev) ? c->dl[l + 1].diag : nullptr;
         build_level_fp32(L, cdiag, c->mem, c->stream);
     }
-    c->Ainv_s = c->mem.alloc<double>((size_t)c->nL * c->nL);
-    scale_inverse_device(c->nL, c->dl[nlev - 1].diag, c->Ainv, c->Ainv_s, c->stream);
+    if (c->diss.on) {
+        dissect_scaled(c->diss, c->dl[nlev - 1].diag, c->mem, c->stream);
+    } else {
+        c->Ainv_s = c->mem.alloc<double>((size_t)c->nL * c->nL);
+        scale_inverse_device(c->nL, c->dl[nlev - 1].diag, c->Ainv, c->Ainv_s, c->stream);
+    }
     if (c->p.coarsest_fp32) {
         c->ld32 = (c->nL + 3) & ~3;
         c->Ainv_s32 = c->mem.alloc<float>((size_t)c->nL * c->ld32);
@@ -874,14 +885,14 @@ double autotune_shapes(amg_ctx* c) {
         const int rule = shape_of(L);
         double t_rule = 1e30, t_best = 1e30;
         int best = rule;
+        std::vector<int> tries = {kStaged, 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4, 4 | kHalfBlock, 8,
+                                  8 | kHalfBlock, 2 | kSweep, 2 | kHalfBlock | kSweep, 4 | kSweep,
+                                  4 | kHalfBlock | kSweep, 8 | kSweep, 8 | kHalfBlock | kSweep};
         // staged kernels also with a smaller shared-memory carveout (percent
         // of the maximum 228 KB: 100, 132 or 164 KB), leaving more L1 for the
         // neighbour gathers
-        std::vector<int> tries = {kStaged, with_carve(kStaged, 44), with_carve(kStaged, 58),
-                                  with_carve(kStaged, 72), 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4,
-                                  4 | kHalfBlock, 8, 8 | kHalfBlock, 2 | kSweep,
-                                  2 | kHalfBlock | kSweep, 4 | kSweep, 4 | kHalfBlock | kSweep,
-                                  8 | kSweep, 8 | kHalfBlock | kSweep};
+        if (uses_shared_memory(L))
+            for (int pct : {44, 58, 72}) tries.push_back(with_carve(kStaged, pct));
         // the tail, where every level below is in it
         if (L.split && (l == nlev - 2 || c->tail_l0 <= l + 1) &&
             tail_fits(c, l, c->precision == AMG_FP32_IN_FP64))
@@ -1595,6 +1606,36 @@ void init_device_pool(int device) {
     });
 }
 
+// The dissection of the coarsest matrix where its solve reads less than half of
+// the whole inverse (empty: the dense inverse).  Below 2,000 rows the dense
+// product is a few microseconds and three launches would cost as much; the
+// float32 copy of coarsest_fp32 stays the dense inverse.
+Dissection coarsest_dissection(const HostCsr& A, const amg_params& p) {
+    Dissection none;
+    if (A.n < 2000 || p.coarsest_fp32) return none;
+    int depth = 1;
+    while ((A.n >> depth) > 700) ++depth;
+    Dissection d = dissect(A, depth);
+    const int np = d.parts();
+    const double ns = A.n - d.ptr[np];
+    std::vector<int32_t> part(A.n, -1);
+    double work = ns * ns;
+    for (int k = 0; k < np; ++k) {
+        const double m = d.ptr[k + 1] - d.ptr[k];
+        work += m * m;
+        for (int32_t q = d.ptr[k]; q < d.ptr[k + 1]; ++q) part[d.order[q]] = k;
+    }
+    std::vector<int32_t> seen(np, -1);
+    for (int32_t q = d.ptr[np]; q < A.n; ++q)
+        for (int32_t e = A.rp[d.order[q]]; e < A.rp[d.order[q] + 1]; ++e) {
+            const int k = part[A.ci[e]];
+            if (k < 0 || seen[k] == q) continue;
+            seen[k] = q;
+            work += 2.0 * (d.ptr[k + 1] - d.ptr[k]);
+        }
+    return work < 0.5 * (double)A.n * A.n ? d : none;
+}
+
 void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     NvtxRange nvtx("amg_setup");
     if (!A || !prm || !out) throw Error{AMG_EINVAL, "null argument"};
@@ -1696,10 +1737,13 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
 
     // smoothing orders, bottom-up
     const double t_dev0 = now_ms();
+    Dissection diss;
     {
         std::vector<int32_t>& pl = c->hl[nlev - 1].perm;
         pl.resize(c->nL);
         std::iota(pl.begin(), pl.end(), 0);
+        diss = coarsest_dissection(c->hl[nlev - 1].A, *prm);
+        for (int32_t k = 0; k < (int32_t)diss.order.size(); ++k) pl[diss.order[k]] = k;
         for (int l = nlev - 2; l >= 0; --l) c->hl[l].perm = smoothing_order(c->hl[l]);
     }
     c->dl.resize(nlev);
@@ -1765,10 +1809,16 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
         if (L.nrp) L.rptr_host = rptr;
     }
     // coarsest level: dense inverse
-    c->Ainv = c->mem.alloc<double>((size_t)c->nL * c->nL);
     const double t_inv0 = now_ms();
     NvtxRange nvtx_inv("coarsest inverse");
-    if (!dense_inverse_device(dA[nlev - 1], c->Ainv, s))
+    bool spd;
+    if (!diss.order.empty()) {
+        spd = dissect_device(c->hl[nlev - 1].A, diss, c->mem, c->diss, s);
+    } else {
+        c->Ainv = c->mem.alloc<double>((size_t)c->nL * c->nL);
+        spd = dense_inverse_device(dA[nlev - 1], c->Ainv, s);
+    }
+    if (!spd)
         throw Error{AMG_ENOTSPD, "coarsest matrix is not positive definite"};
     const double inverse_ms = now_ms() - t_inv0;
 
