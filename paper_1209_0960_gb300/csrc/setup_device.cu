@@ -192,35 +192,50 @@ constexpr int kPanel = 32;
 // one thread per entry (32 x 32 threads); write L_kk back (upper part zero)
 // and D = L_kk^-1 to Dk (32 x 32, row-major).  A pivot <= 0 sets *err and
 // continues with 1.
+//
+// A warp-wide float64 operation takes 64 cycles of a sub-partition whatever
+// its active lanes, and a division about twenty of them.  Dividing a column by
+// its pivot with one thread in each of the 32 warps took 5 us a column; here
+// one thread forms the pivot's square root and reciprocal, and a column is one
+// warp's multiplication.  The inverse of 275 rows: 1.96 -> 1.59 ms (0.96 with the
+// smaller output tiles, see invert_dense).
 __global__ void __launch_bounds__(kPanel * kPanel) k_potrf_block(int n, int k0, double* __restrict__ W,
                                                                  double* __restrict__ Dk,
                                                                  int* __restrict__ err) {
     __shared__ double T[kPanel][kPanel + 1];
     __shared__ double Y[kPanel][kPanel + 1];
+    __shared__ double rinv[kPanel];
     const int r = threadIdx.x / kPanel, c = threadIdx.x % kPanel;
     const int m = min(kPanel, n - k0);
     T[r][c] = (r < m && c <= r) ? W[(size_t)(k0 + r) * n + k0 + c] : 0.0;
     Y[r][c] = (r == c && r < m) ? 1.0 : 0.0;
     __syncthreads();
-    // right-looking Cholesky: column j, then the rank-1 update of the rest
+    // right-looking Cholesky: column j (by the first warp, lane = row), then
+    // the rank-1 update of the rest
     for (int j = 0; j < m; ++j) {
-        if (r == j && c == j) {
-            double d = T[j][j];
-            if (!(d > 0.0)) {
-                *err = 1;
-                d = 1.0;
+        if (r == 0) {
+            double inv = 0.0;
+            if (c == 0) {
+                double d = T[j][j];
+                if (!(d > 0.0)) {
+                    *err = 1;
+                    d = 1.0;
+                }
+                const double root = sqrt(d);
+                T[j][j] = root;
+                inv = 1.0 / root;
+                rinv[j] = inv;
             }
-            T[j][j] = sqrt(d);
+            inv = __shfl_sync(0xffffffffu, inv, 0);
+            if (c > j && c < m) T[c][j] *= inv;
         }
-        __syncthreads();
-        if (c == j && r > j && r < m) T[r][j] /= T[j][j];
         __syncthreads();
         if (r > j && r < m && c > j && c <= r) T[r][c] -= T[r][j] * T[c][j];
         __syncthreads();
     }
     // D = L_kk^-1 by forward elimination on the identity, row j at a time
     for (int j = 0; j < m; ++j) {
-        if (r == j && c <= j) Y[j][c] /= T[j][j];
+        if (r == j && c <= j) Y[j][c] *= rinv[j];
         __syncthreads();
         if (r > j && r < m && c <= j) Y[r][c] -= T[r][j] * Y[j][c];
         __syncthreads();
@@ -259,39 +274,41 @@ __device__ __forceinline__ void tri_pair(int b, int& I, int& J) {
 }
 
 // Trailing update W[i][j] -= sum_t P[i][t] P[j][t] over the lower tiles of
-// rows/columns >= r0 (P = the panel W[:, k0:k0+m]); 64 x 64 tiles, 256
-// threads, 4 x 4 outputs per thread.
+// rows/columns >= r0 (P = the panel W[:, k0:k0+m]); TS x TS tiles, 256
+// threads, TS/16 x TS/16 outputs per thread.
+template <int TS>
 __global__ void __launch_bounds__(256) k_syrk(int n, int r0, int k0, int m, double* __restrict__ W) {
-    __shared__ double Pa[64][kPanel + 1];
-    __shared__ double Pb[64][kPanel + 1];
+    constexpr int TU = TS / 16;
+    __shared__ double Pa[TS][kPanel + 1];
+    __shared__ double Pb[TS][kPanel + 1];
     int I, J;
     tri_pair((int)blockIdx.x, I, J);
-    const int i0 = r0 + 64 * I, j0 = r0 + 64 * J;
-    for (int t = threadIdx.x; t < 64 * kPanel; t += blockDim.x) {
+    const int i0 = r0 + TS * I, j0 = r0 + TS * J;
+    for (int t = threadIdx.x; t < TS * kPanel; t += blockDim.x) {
         const int r = t / kPanel, q = t % kPanel;
         Pa[r][q] = (i0 + r < n && q < m) ? W[(size_t)(i0 + r) * n + k0 + q] : 0.0;
         Pb[r][q] = (j0 + r < n && q < m) ? W[(size_t)(j0 + r) * n + k0 + q] : 0.0;
     }
     __syncthreads();
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    double acc[4][4] = {};
+    double acc[TU][TU] = {};
     for (int q = 0; q < m; ++q) {
-        double av[4], bv[4];
+        double av[TU], bv[TU];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            av[u] = Pa[ty * 4 + u][q];
-            bv[u] = Pb[tx * 4 + u][q];
+        for (int u = 0; u < TU; ++u) {
+            av[u] = Pa[ty * TU + u][q];
+            bv[u] = Pb[tx * TU + u][q];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < TU; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+            for (int v = 0; v < TU; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < TU; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = i0 + ty * 4 + u, j = j0 + tx * 4 + v;
+        for (int v = 0; v < TU; ++v) {
+            const int i = i0 + ty * TU + u, j = j0 + tx * TU + v;
             if (i < n && j < n && j <= i) W[(size_t)i * n + j] -= acc[u][v];
         }
 }
@@ -323,83 +340,87 @@ __global__ void __launch_bounds__(kPanel * kPanel) k_trinv_final(int n, int i0, 
 }
 
 // Update after block row i0 is final: S_jc += L_j,i Y_i,c for the block rows
-// j > i0 and column tiles c <= i0, 64 x 64 output tiles of (rows >= i0 + m,
-// columns < i0 + m), K = m; 256 threads, 4 x 4 outputs each.
+// j > i0 and column tiles c <= i0, TS x TS output tiles of (rows >= i0 + m,
+// columns < i0 + m), K = m; 256 threads, TS/16 x TS/16 outputs each.
+template <int TS>
 __global__ void __launch_bounds__(256) k_trinv_update(int n, int i0, int m, const double* __restrict__ L,
                                                       double* __restrict__ Y) {
-    __shared__ double Pa[64][kPanel + 1];   // L[j rows, i0 .. i0+m)
-    __shared__ double Pb[kPanel][64 + 1];   // Y[i0 .. i0+m, c columns]
+    constexpr int TU = TS / 16;
+    __shared__ double Pa[TS][kPanel + 1];   // L[j rows, i0 .. i0+m)
+    __shared__ double Pb[kPanel][TS + 1];   // Y[i0 .. i0+m, c columns]
     const int r0 = i0 + m, ncol = i0 + m;
-    const int tiles_c = (ncol + 63) / 64;
+    const int tiles_c = (ncol + TS - 1) / TS;
     const int J = (int)blockIdx.x / tiles_c, C = (int)blockIdx.x % tiles_c;
-    const int j0 = r0 + 64 * J, c0 = 64 * C;
-    for (int t = threadIdx.x; t < 64 * kPanel; t += blockDim.x) {
+    const int j0 = r0 + TS * J, c0 = TS * C;
+    for (int t = threadIdx.x; t < TS * kPanel; t += blockDim.x) {
         const int rr = t / kPanel, q = t % kPanel;
         Pa[rr][q] = (j0 + rr < n && q < m) ? L[(size_t)(j0 + rr) * n + i0 + q] : 0.0;
-        const int qq = t / 64, cc = t % 64;
+        const int qq = t / TS, cc = t % TS;
         Pb[qq][cc] = (qq < m && c0 + cc < ncol) ? Y[(size_t)(i0 + qq) * n + c0 + cc] : 0.0;
     }
     __syncthreads();
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    double acc[4][4] = {};
+    double acc[TU][TU] = {};
     for (int q = 0; q < m; ++q) {
-        double av[4], bv[4];
+        double av[TU], bv[TU];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            av[u] = Pa[ty * 4 + u][q];
-            bv[u] = Pb[q][tx * 4 + u];
+        for (int u = 0; u < TU; ++u) {
+            av[u] = Pa[ty * TU + u][q];
+            bv[u] = Pb[q][tx * TU + u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < TU; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+            for (int v = 0; v < TU; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < TU; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int j = j0 + ty * 4 + u, cc = c0 + tx * 4 + v;
+        for (int v = 0; v < TU; ++v) {
+            const int j = j0 + ty * TU + u, cc = c0 + tx * TU + v;
             if (j < n && cc < ncol) Y[(size_t)j * n + cc] += acc[u][v];
         }
 }
 
-// X = Y^T Y for the lower tiles (I >= J) of 64 x 64, mirrored to the upper
-// part: X[i][j] = sum_{k >= 64 I} Y[k][i] Y[k][j] (Y is lower triangular).
+// X = Y^T Y for the lower tiles (I >= J) of TS x TS, mirrored to the upper
+// part: X[i][j] = sum_{k >= TS I} Y[k][i] Y[k][j] (Y is lower triangular).
+template <int TS>
 __global__ void __launch_bounds__(256) k_yty(int n, const double* __restrict__ Y, double* __restrict__ X) {
-    __shared__ double Ya[kPanel][64 + 1];
-    __shared__ double Yb[kPanel][64 + 1];
+    constexpr int TU = TS / 16;
+    __shared__ double Ya[kPanel][TS + 1];
+    __shared__ double Yb[kPanel][TS + 1];
     int I, J;
     tri_pair((int)blockIdx.x, I, J);
-    const int i0 = 64 * I, j0 = 64 * J;
+    const int i0 = TS * I, j0 = TS * J;
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    double acc[4][4] = {};
+    double acc[TU][TU] = {};
     for (int k0 = i0; k0 < n; k0 += kPanel) {
-        for (int t = threadIdx.x; t < kPanel * 64; t += blockDim.x) {
-            const int kk = t / 64, c = t % 64;
+        for (int t = threadIdx.x; t < kPanel * TS; t += blockDim.x) {
+            const int kk = t / TS, c = t % TS;
             const bool ok = k0 + kk < n;
             Ya[kk][c] = (ok && i0 + c < n) ? Y[(size_t)(k0 + kk) * n + i0 + c] : 0.0;
             Yb[kk][c] = (ok && j0 + c < n) ? Y[(size_t)(k0 + kk) * n + j0 + c] : 0.0;
         }
         __syncthreads();
         for (int q = 0; q < kPanel; ++q) {
-            double av[4], bv[4];
+            double av[TU], bv[TU];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                av[u] = Ya[q][ty * 4 + u];
-                bv[u] = Yb[q][tx * 4 + u];
+            for (int u = 0; u < TU; ++u) {
+                av[u] = Ya[q][ty * TU + u];
+                bv[u] = Yb[q][tx * TU + u];
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < TU; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
+                for (int v = 0; v < TU; ++v) acc[u][v] = fma(av[u], bv[v], acc[u][v]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < TU; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = i0 + ty * 4 + u, j = j0 + tx * 4 + v;
+        for (int v = 0; v < TU; ++v) {
+            const int i = i0 + ty * TU + u, j = j0 + tx * TU + v;
             if (i < n && j < n && j <= i) {
                 X[(size_t)i * n + j] = acc[u][v];
                 X[(size_t)j * n + i] = acc[u][v];
@@ -629,7 +650,8 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
 }
 
 // Minv = W^-1 for the dense matrix whose lower triangle is W (overwritten)
-static bool invert_dense(int n, double* W, double* Minv, cudaStream_t s) {
+template <int TS>
+static bool invert_dense_tiles(int n, double* W, double* Minv, cudaStream_t s) {
     const int np = (n + kPanel - 1) / kPanel;
     DevArena tmp(s);
     double* Y = tmp.alloc<double>((size_t)n * n);
@@ -644,8 +666,8 @@ static bool invert_dense(int n, double* W, double* Minv, cudaStream_t s) {
         if (r0 < n) {
             k_panel<<<blocks_for((int64_t)(n - r0) * 32), kBlock, 0, s>>>(n, k0, m, W,
                                                                            D + (size_t)p * kPanel * kPanel);
-            const int t = (n - r0 + 63) / 64;
-            k_syrk<<<t * (t + 1) / 2, 256, 0, s>>>(n, r0, k0, m, W);
+            const int t = (n - r0 + TS - 1) / TS;
+            k_syrk<TS><<<t * (t + 1) / 2, 256, 0, s>>>(n, r0, k0, m, W);
         }
     }
     // Y = L^-1 (Y starts at zero: the running sums), then M^-1 = Y^T Y
@@ -653,17 +675,25 @@ static bool invert_dense(int n, double* W, double* Minv, cudaStream_t s) {
         const int i0 = p * kPanel, m = std::min(kPanel, n - i0), r0 = i0 + m;
         k_trinv_final<<<p + 1, kPanel * kPanel, 0, s>>>(n, i0, m, Y, D + (size_t)p * kPanel * kPanel);
         if (r0 < n) {
-            const int tiles = ((n - r0 + 63) / 64) * ((r0 + 63) / 64);
-            k_trinv_update<<<tiles, 256, 0, s>>>(n, i0, m, W, Y);
+            const int tiles = ((n - r0 + TS - 1) / TS) * ((r0 + TS - 1) / TS);
+            k_trinv_update<TS><<<tiles, 256, 0, s>>>(n, i0, m, W, Y);
         }
     }
-    const int t = (n + 63) / 64;
-    k_yty<<<t * (t + 1) / 2, 256, 0, s>>>(n, Y, Minv);
+    const int t = (n + TS - 1) / TS;
+    k_yty<TS><<<t * (t + 1) / 2, 256, 0, s>>>(n, Y, Minv);
     AMG_CUDA_TRY(cudaGetLastError());
     int herr = 0;
     AMG_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
     return herr == 0;
+}
+
+// Output tiles of 64 x 64, or of 32 x 32 where those would leave most SMs idle: a
+// tile's float64 work runs at one SM's two multiply-adds a clock, 300 us for the
+// last product of a 64 x 64 tile at 275 rows (whose inverse took 1.59 ms, and takes
+// 0.96).
+static bool invert_dense(int n, double* W, double* Minv, cudaStream_t s) {
+    return n < 1024 ? invert_dense_tiles<32>(n, W, Minv, s) : invert_dense_tiles<64>(n, W, Minv, s);
 }
 
 bool dense_inverse_device(const DevCsr& A, double* Minv, cudaStream_t s) {
