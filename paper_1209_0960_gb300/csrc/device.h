@@ -719,6 +719,10 @@ struct amg_ctx {
     cudaGraphExec_t graph_a[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t graph_b[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     std::vector<cudaGraphExec_t> graph_from[2];   // V-cycle from level l (profiling), per precision
+    // z = B r on the level-0 vectors for amg_vcycle, per precision, built by its
+    // second call with the current shapes (vcycle_calls)
+    cudaGraphExec_t graph_v[2] = {nullptr, nullptr};
+    int vcycle_calls[2] = {0, 0};
     // the whole iteration loop as one graph with a device-side WHILE node,
     // [precision][flexible]; solve_graph_state 0 = not built yet, 1 = built,
     // -1 = the runtime refused it (the host-driven loop runs instead)
@@ -790,9 +794,11 @@ struct amg_ctx {
                 if (graph_b[a][b]) cudaGraphExecDestroy(graph_b[a][b]);
                 if (graph_solve[a][b]) cudaGraphExecDestroy(graph_solve[a][b]);
             }
-        for (int a = 0; a < 2; ++a)
+        for (int a = 0; a < 2; ++a) {
             for (cudaGraphExec_t g : graph_from[a])
                 if (g) cudaGraphExecDestroy(g);
+            if (graph_v[a]) cudaGraphExecDestroy(graph_v[a]);
+        }
         if (ev_in) cudaEventDestroy(ev_in);
         if (ev_out) cudaEventDestroy(ev_out);
         mem.release();   // stream-ordered frees, before the stream goes away

@@ -585,6 +585,9 @@ void drop_graphs(amg_ctx* c) {
             c->solve_graph_state[a][b] = 0;
         }
         c->vrec_ok[a] = false;
+        if (c->graph_v[a]) cudaGraphExecDestroy(c->graph_v[a]);
+        c->graph_v[a] = nullptr;
+        c->vcycle_calls[a] = 0;
         if (c->graph_bi[a]) cudaGraphExecDestroy(c->graph_bi[a]);
         c->graph_bi[a] = nullptr;
         c->bi_graph_state[a] = 0;
@@ -1885,6 +1888,30 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     *out = c.release();
 }
 
+// The V-cycle of amg_vcycle as one graph on the context's own vectors: launching
+// its kernels one by one costs the host about 4.5 us each, more than most of
+// them take (128^3: 88 launches, 437 us a call against 385 us in a graph).  Built
+// by the second call, so that a context that applies its V-cycle once does not
+// pay for it, for V-cycles of 40 launches and more (64x64: 9 launches take 53 us,
+// in a graph 55); not while the launches are profiled, nor inside a capture of
+// the caller's.
+cudaGraphExec_t vcycle_graph(amg_ctx* c) {
+    const int pr = c->precision;
+    if (!cg_graphs(c) || c->prof.graphs) return nullptr;
+    int launches = 0;
+    for (int l = 0; l + 1 < (int)c->dl.size() && l < c->tail_l0; ++l) launches += 4 * c->dl[l].ncolours + 1;
+    if (launches < 40) return nullptr;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    AMG_CUDA_TRY(cudaStreamIsCapturing(c->stream, &st));
+    if (st != cudaStreamCaptureStatusNone) return nullptr;
+    if (c->vcycle_calls[pr] < 1) {
+        ++c->vcycle_calls[pr];
+        return nullptr;
+    }
+    if (!c->graph_v[pr]) c->graph_v[pr] = capture_graph(c, [&] { precondition(c, c->r, c->z); });
+    return c->graph_v[pr];
+}
+
 }  // namespace
 }  // namespace amg
 
@@ -1956,9 +1983,17 @@ int amg_vcycle(amg_ctx* c, const double* r_dev, double* z_dev) {
         if (!c || !r_dev || !z_dev) throw Error{AMG_EINVAL, "null argument"};
         const int n = c->dl[0].n;
         enter(c);
-            launch_scatter(n, c->perm0, r_dev, c->r, c->stream);
-        precondition(c, c->r, c->z);
+        launch_scatter(n, c->perm0, r_dev, c->r, c->stream);
+        if (cudaGraphExec_t g = vcycle_graph(c)) {
+            AMG_CUDA_TRY(cudaGraphLaunch(g, c->stream));
+            // a programmatic dependent launch does not wait for a graph before it:
+            // the gather starts in plain stream order
+            t_launch_overlap = false;
+        } else {
+            precondition(c, c->r, c->z);
+        }
         launch_gather(n, c->perm0, c->z, z_dev, c->stream);
+        t_launch_overlap = c->p.launch_overlap != 0;
         AMG_CUDA_TRY(cudaGetLastError());
         leave(c);
     });
