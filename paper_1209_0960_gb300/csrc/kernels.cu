@@ -32,13 +32,6 @@ namespace {
 // ---------------------------------------------------------------------------
 // helpers
 // ---------------------------------------------------------------------------
-// load of setup-time per-row data (length, diagonal): evict-first on the
-// streamed fine level
-template <bool STREAM, typename T>
-__device__ __forceinline__ T ldm(const T* p) {
-    return STREAM ? __ldcs(p) : *p;
-}
-
 // acc + sgn * sum_k A_row,k x_col(k) over the stored off-diagonal entries of a
 // SELL-32 row (base = slice start + row mod 32)
 template <bool NEG, typename T, typename X>
@@ -293,8 +286,8 @@ __device__ __forceinline__ T nbr_value(int j, const T* x, const T* b, const T* _
 // neighbour values are read after pdl_wait().  With several lanes per row the
 // first batch of column indices and values (setup-time data) is loaded before
 // it, so those loads overlap the predecessor kernel.
-// LPR = lanes per row (1, 2, 4 or 8).  The fine level has kernels of its own
-// (below), with the matrix staged in shared memory.
+// LPR = lanes per row (1, 2, 4 or 8).  One row per thread with the matrix staged
+// in shared memory, or a whole row in registers, has kernels of its own (below).
 constexpr int kFine = 0;
 template <int LPR>
 __host__ __device__ constexpr int lanes_of() { return LPR == kFine ? 1 : LPR; }
@@ -823,8 +816,10 @@ __global__ void __launch_bounds__(kBlock) k_sweep(int npass, const SweepPass* __
 }
 
 // ---------------------------------------------------------------------------
-// Fine-level kernels: the matrix staged in shared memory by the bulk-copy
-// engine.
+// Staged kernels (lanes per row 0): the matrix staged in shared memory by the
+// bulk-copy engine.  A fine level of a 5-point or 7-point stencil reads its rows
+// into registers instead (WideRow); these run on fine levels of other widths,
+// and on coarse levels where the tuner or a caller picks them.
 //
 // A block of kBlock threads owns kBlock / 32 consecutive slices, one row per
 // thread.  Those slices are contiguous in scol and sval, so one thread starts
