@@ -549,11 +549,9 @@ def measure_workload(args, dist, workload, grid, steps, warmup, headline, kernel
                            "bytes_per_launch": per_b, "ms_per_launch": per_ms,
                            "share_of_solve": top["total_ms"] / sum(d["total_ms"] for d in prof64),
                            "traffic": kernel_traffic(top["name"], workload)}
-        # kernels in the timed region: the profiled solve's launches (host-driven
-        # loop) plus one loop-condition kernel per iteration of the device loop
+        # kernels in the timed region: the profiled solve's launches (the device
+        # loop runs the same kernels as the profiled, host-driven one)
         launches = sum(d["launches"] for d in prof64 if d["name"] != "zero")
-        if i64.get("device_loop"):
-            launches += i64["iterations"]
         rec["gpu_launches"] = launches * steps
         rec["clocks"] = clk
         rec["device_loop"] = i64.get("device_loop")

@@ -115,6 +115,13 @@ struct PcgScalars {
     int32_t loops;    // device-side loop: conditions evaluated (a bound of its own)
 };
 
+// The condition of a device-side loop, set by the kernel that ends an iteration
+// (on = 0: none).
+struct LoopCond {
+    cudaGraphConditionalHandle h = 0;
+    int32_t on = 0;
+};
+
 // Scalars of the BiCGSTAB recurrence, resident on the device.
 struct BiScalars {
     double r0;        // ||r_0||
@@ -379,7 +386,6 @@ struct CgWork {
 // Sets the condition of the device-side CG loop (a WHILE graph node) to
 // "not converged, no breakdown, fewer than maxit iterations" from the device
 // scalars; it also counts its own evaluations and stops at maxit.
-void launch_cg_continue(cudaGraphConditionalHandle h, PcgScalars* sc, cudaStream_t s);
 extern thread_local bool t_launch_overlap;
 // grids above this many blocks: CG kernels launch without the overlap (a wide
 // grid that starts early only occupies the SMs its predecessor is still
@@ -560,7 +566,15 @@ void launch_cg_residual(const DevLevel& L, const double* b, const double* x, dou
                         CgWork& w, int mode, double* out, cudaStream_t s);
 void launch_cg_spmv_pq(const DevLevel& L, const double* p, double* q, CgWork& w, cudaStream_t s);
 void launch_cg_update(int n, double* x, double* r, const double* p, const double* q, CgWork& w,
-                      cudaStream_t s);
+                      LoopCond cond, cudaStream_t s);
+// The work of an iteration outside the V-cycle as one cluster, on systems of up to
+// kCgClusterRows rows: 16 SMs have a tenth of the device's float64 rate, so that it
+// gains 5 us an iteration at 4,096 rows, 3.6 at 24,000, and at 32,800 nothing (one
+// of two workloads slower).
+constexpr int kCgThreads = 512, kCgBlocks = 16, kCgClusterRows = 24576;
+bool cg_cluster_fits(const DevLevel& L);
+void launch_cg_cluster(const DevLevel& L, double* r, const double* z, double* zold, double* p, double* q,
+                       double* x, CgWork& w, LoopCond cond, cudaStream_t s);
 void launch_cg_rz(int n, const double* r, const double* z, const double* zold, double* p,
                   CgWork& w, int mode, cudaStream_t s);
 void launch_cg_p(int n, const double* z, double* p, double* zold, const CgWork& w,
@@ -583,8 +597,8 @@ void launch_bi_half(int n, const double* r, const double* v, double* sv, CgWork&
                     BiScalars* bs, cudaStream_t s);
 void launch_bi_update(int n, double* x, const double* y, const double* z, const double* sv,
                       const double* t, double* r, const double* rt, CgWork& wk, BiScalars* bs,
-                      cudaStream_t s);
-void launch_bi_continue(cudaGraphConditionalHandle h, BiScalars* bs, cudaStream_t s);
+                      LoopCond cond, cudaStream_t s);
+void launch_bi_continue(LoopCond cond, BiScalars* bs, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // setup on the device (setup_device.cu)
@@ -719,6 +733,7 @@ struct amg_ctx {
     cudaGraphExec_t graph_a[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t graph_b[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     std::vector<cudaGraphExec_t> graph_from[2];   // V-cycle from level l (profiling), per precision
+    bool cg_cluster = false;   // CG outside the V-cycle as one cluster launch
     // z = B r on the level-0 vectors for amg_vcycle, per precision, built by its
     // second call with the current shapes (vcycle_calls)
     cudaGraphExec_t graph_v[2] = {nullptr, nullptr};

@@ -36,7 +36,7 @@ namespace {
 // SELL-32 row (base = slice start + row mod 32)
 template <bool NEG, typename T, typename X>
 __device__ __forceinline__ T sell_row(int64_t base, int len, const int32_t* __restrict__ scol,
-                                      const T* __restrict__ sval, const X* x, T acc, int n,
+                                      const T* __restrict__ sval, const X& x, T acc, int n,
                                       int32_t* err) {
 #pragma unroll 4
     for (int k = 0; k < len; ++k) {
@@ -73,8 +73,8 @@ struct WideRow {
     }
     // acc +- sum over the entries (ALL, or those with j < jmax) of a x_j, in
     // stored order
-    template <bool NEG, bool ALL>
-    __device__ __forceinline__ T add(const T* x, T acc, int jmax, int n, int32_t* err) const {
+    template <bool NEG, bool ALL, typename X>
+    __device__ __forceinline__ T add(const X& x, T acc, int jmax, int n, int32_t* err) const {
         T v[W];
 #pragma unroll
         for (int k = 0; k < W; ++k) v[k] = (!kChecks || (k < len && index_ok(j[k], n, err))) ? x[j[k]] : T(0);
@@ -102,14 +102,14 @@ struct RowLoop {
     const double* __restrict__ diag;
     WideRow<double, W> cur;
     int row, step;
-    __device__ __forceinline__ RowLoop(int n_, int64_t sw_, const uint16_t* rlen_, const int32_t* scol_,
-                                       const double* sval_, const double* diag_)
-        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_),
-          row(blockIdx.x * blockDim.x + threadIdx.x), step(gridDim.x * blockDim.x) {
+    __device__ __forceinline__ RowLoop(int first, int n_, int64_t sw_, const uint16_t* rlen_,
+                                       const int32_t* scol_, const double* sval_, const double* diag_)
+        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_), row(first),
+          step(gridDim.x * blockDim.x) {
         cur.load(row, row < n, sw, rlen, scol, sval, diag);
     }
-    template <bool NEG, typename Start, typename Done>
-    __device__ __forceinline__ void run(const double* x, int32_t* err, Start start, Done done) {
+    template <bool NEG, typename X, typename Start, typename Done>
+    __device__ __forceinline__ void run(const X& x, int32_t* err, Start start, Done done) {
         while (row < n) {
             const int64_t after = (int64_t)row + step;
             WideRow<double, W> next;
@@ -129,12 +129,13 @@ struct RowLoop<0> {
     const int32_t* __restrict__ scol;
     const double* __restrict__ sval;
     const double* __restrict__ diag;
-    __device__ __forceinline__ RowLoop(int n_, int64_t sw_, const uint16_t* rlen_, const int32_t* scol_,
-                                       const double* sval_, const double* diag_)
-        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_) {}
-    template <bool NEG, typename Start, typename Done>
-    __device__ __forceinline__ void run(const double* x, int32_t* err, Start start, Done done) {
-        for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
+    int row;
+    __device__ __forceinline__ RowLoop(int first, int n_, int64_t sw_, const uint16_t* rlen_,
+                                       const int32_t* scol_, const double* sval_, const double* diag_)
+        : n(n_), sw(sw_), rlen(rlen_), scol(scol_), sval(sval_), diag(diag_), row(first) {}
+    template <bool NEG, typename X, typename Start, typename Done>
+    __device__ __forceinline__ void run(const X& x, int32_t* err, Start start, Done done) {
+        for (; row < n; row += gridDim.x * blockDim.x) {
             const int64_t base = (int64_t)(row >> 5) * sw + (row & 31);
             done(row, sell_row<NEG>(base, __ldcs(rlen + row), scol, sval, x, start(row, __ldcs(diag + row)),
                                     n, err));
@@ -158,36 +159,10 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 
-// Called by every block after it has a block sum (in thread 0).  The last
-// block to arrive combines all partial sums in index order and applies the
-// CG scalar update of `mode`.
-__device__ void finish_reduction(double v0, double v1, double* partials, double* partials2,
-                                 unsigned int* counter, PcgScalars* sc, double* out, int mode,
-                                 double* sh);
 __device__ __forceinline__ bool finite_dot(double a) { return isfinite(a); }
 
-__device__ void finish_reduction(double v0, double v1, double* partials, double* partials2,
-                                 unsigned int* counter, PcgScalars* sc, double* out, int mode,
-                                 double* sh) {
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = v0;
-        if (mode == kRZFlex) partials2[blockIdx.x] = v1;
-        __threadfence();
-        unsigned int t = atomicAdd(counter, 1u);
-        last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last) return;
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        a += __ldcg(partials + i);
-        if (mode == kRZFlex) b += __ldcg(partials2 + i);
-    }
-    a = block_sum(a, sh);
-    if (mode == kRZFlex) b = block_sum(b, sh);
-    if (threadIdx.x != 0) return;
-    *counter = 0u;
+// The CG scalar update of `mode` from its sums a (and b, kRZFlex).
+__device__ void cg_scalars(int mode, double a, double b, PcgScalars* sc, double* out) {
     // a NaN or infinity in a dot product of the iteration ends the solve
     if (mode != kStore && (!finite_dot(a) || (mode == kRZFlex && !finite_dot(b)))) {
         if (mode == kRR0) {
@@ -240,13 +215,45 @@ __device__ void finish_reduction(double v0, double v1, double* partials, double*
     }
 }
 
-// Condition of the device-side PCG loop, evaluated after each x/r update:
-// continue while ||r|| > tol ||r_0||, p.Ap > 0 and fewer than maxit
-// iterations.  The evaluation count is a second, independent bound.
-__global__ void k_cg_continue(cudaGraphConditionalHandle h, PcgScalars* sc) {
+// Called by every block after it has a block sum (in thread 0).  The last
+// block to arrive combines all partial sums in index order and applies the
+// CG scalar update of `mode`; true in the thread that did.
+__device__ bool finish_reduction(double v0, double v1, double* partials, double* partials2,
+                                 unsigned int* counter, PcgScalars* sc, double* out, int mode,
+                                 double* sh) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = v0;
+        if (mode == kRZFlex) partials2[blockIdx.x] = v1;
+        __threadfence();
+        unsigned int t = atomicAdd(counter, 1u);
+        last = (t == gridDim.x - 1);
+    }
+    __syncthreads();
+    if (!last) return false;
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        a += __ldcg(partials + i);
+        if (mode == kRZFlex) b += __ldcg(partials2 + i);
+    }
+    a = block_sum(a, sh);
+    if (mode == kRZFlex) b = block_sum(b, sh);
+    if (threadIdx.x != 0) return false;
+    *counter = 0u;
+    cg_scalars(mode, a, b, sc, out);
+    return true;
+}
+
+// Condition of the device-side PCG loop, evaluated after each x/r update by the
+// thread that ended it: continue while ||r|| > tol ||r_0||, p.Ap > 0 and fewer
+// than maxit iterations.  The evaluation count is a second, independent bound.
+// (As a kernel of its own after the update it made the loop 4 to 7 us an
+// iteration longer: 64x64 Poisson 73 -> 69 us, 61x47x70 mixed 148 -> 142.)
+__device__ __forceinline__ void cg_continue(const LoopCond& cond, PcgScalars* sc) {
+    if (!cond.on) return;
     const int32_t loops = ++sc->loops;
     const bool go = sc->done == 0 && sc->status == 0 && sc->iters < sc->maxit && loops < sc->maxit;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
+    cudaGraphSetConditional(cond.h, go ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -481,7 +488,10 @@ struct ResidualBody {
 // (see RowPart): the backward passes read the upper parts only, the forward
 // passes from a zero guess and the residual the lower parts only.  The passes
 // of a coarse level are bound by their gathers of x and by the float64 pipe,
-// both of which shrink with the entries.
+// both of which shrink with the entries.  Split against whole rows: V-cycle
+// 64x64 109 -> 90 us and 128^3 504 -> 479 us, solves 81x64x77 6.01 -> 5.25 ms
+// and anisotropic 256x224x209 mixed 336 -> 305 ms.  With two colours (the fine
+// level) the parts of a row are all or nothing and nothing is gained.
 // ---------------------------------------------------------------------------
 
 // entries per lane of one batch of a row part
@@ -1177,7 +1187,8 @@ struct FineSplitResidualBody {
 // Adds the sum of the values v of each run of equal keys in the warp (key -1:
 // none; equal keys are consecutive lanes) to bc[key].  Doubling steps, as many
 // as the longest run needs: two or three float64 additions a warp where a walk
-// along the run took one per row.
+// along the run took one per row.  (With the rows in registers the fine level of
+// 128^3 went 164 -> 143 us a V-cycle in float64, 136 -> 118 in float32.)
 template <typename T>
 __device__ __forceinline__ void restrict_runs(T v, int key, T* bc) {
     const int lane = threadIdx.x & 31;
@@ -1684,7 +1695,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_residual(int n, int64_t sw,
                                                         double* out, int mode) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
-    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
+    RowLoop<W> rows(blockIdx.x * blockDim.x + threadIdx.x, n, sw, rlen, scol, sval, diag);
     pdl_wait();
     double acc = 0.0;
     rows.template run<true>(
@@ -1709,7 +1720,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_spmv_pq(int n, int64_t sw,
                                                        unsigned int* counter, PcgScalars* sc) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
-    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
+    RowLoop<W> rows(blockIdx.x * blockDim.x + threadIdx.x, n, sw, rlen, scol, sval, diag);
     pdl_wait();
     double acc = 0.0, pi = 0.0;
     rows.template run<false>(
@@ -1732,7 +1743,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_update(int n, double* __restrict_
                                                       const double* __restrict__ p,
                                                       const double* __restrict__ q,
                                                       double* partials, unsigned int* counter,
-                                                      PcgScalars* sc) {
+                                                      PcgScalars* sc, const LoopCond cond) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
     pdl_wait();
@@ -1762,7 +1773,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_update(int n, double* __restrict_
         acc = fmad(v, v, acc);
     }
     const double t = block_sum(acc, sh);
-    finish_reduction(t, 0.0, partials, nullptr, counter, sc, nullptr, kRR, sh);
+    if (finish_reduction(t, 0.0, partials, nullptr, counter, sc, nullptr, kRR, sh)) cg_continue(cond, sc);
 }
 
 // rho = r.z (and, flexible, r.(z - z_old)) -> beta; mode kRho0 sets p = z too
@@ -1831,6 +1842,123 @@ __global__ void __launch_bounds__(kBlock) k_cg_p(int n, const double* __restrict
     }
 }
 
+// Sum of v over the cluster's threads, in every lane of warp 0 of every block and
+// with the same bits in all of them.  One cluster barrier, which also orders the
+// blocks' memory accesses before the call before those after it.  any: whether the
+// warp has a value (else v is zero).  slot: used for this sum only.
+__device__ __forceinline__ double cluster_sum(double v, bool any, double* sh, double* slot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (any) v = group_sum<32>(v);
+    if (lane == 0) sh[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        const double t = group_sum<32>(lane < kCgThreads / 32 ? sh[lane] : 0.0);
+        if (lane < kCgBlocks) st_cluster(map_rank(smem_u32(slot + cluster_rank()), (uint32_t)lane), t);
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    return warp == 0 ? group_sum<32>(lane < kCgBlocks ? slot[lane] : 0.0) : 0.0;
+}
+
+// Reads that see what other blocks of the cluster stored before the barrier.
+struct FromL2 {
+    const double* p;
+    __device__ __forceinline__ double operator[](int j) const { return __ldcg(p + j); }
+};
+
+// The work of a CG iteration outside the V-cycle as one cluster: rho = r.z, beta,
+// p, q = A p, alpha, x, r, ||r||^2 and the loop condition; in the first iteration
+// (none counted yet) p = z.  On a system of a few thousand rows each of the five
+// launches this replaces is latency: its start, one trip to L2 for its vectors
+// and two for the last block's sum.  Here a dot product costs a cluster barrier
+// (0.3 us).  A row belongs to one thread throughout, so only p crosses blocks.
+// Bound by that chain (three sums, an exchange of p), not by bytes.  PCG
+// iteration, five launches -> one cluster: 64x64 Poisson 68.9 -> 64.0 us, 90x91
+// 74.4 -> 71.6, 160x150 97.0 -> 93.4, 16x16x17 mixed 38.7 -> 31.7.  (256 threads a
+// block: the same at 4,096 rows, 95.3 at 24,000; rows dealt to the blocks 512 at a
+// time: 65.2 at 4,096, where half the blocks then have none.)
+template <int W>
+__global__ void __launch_bounds__(kCgThreads, 1)
+    k_cg_cluster(int n, int64_t sw, const uint16_t* __restrict__ rlen, const int32_t* __restrict__ scol,
+                 const double* __restrict__ sval, const double* __restrict__ diag, double* r,
+                 const double* z, double* zold, double* p, double* q, double* x, PcgScalars* sc,
+                 const LoopCond cond) {
+    __shared__ double sh[kCgThreads / 32];
+    __shared__ double slot[4][kCgBlocks];
+    __shared__ PcgScalars S;
+    cluster_arrive();
+    pdl_launch_dependents();
+    // warps of 32 rows, dealt to the blocks in turn; warps without rows add
+    // nothing to the sums
+    const int tid = ((int)(threadIdx.x >> 5) * kCgBlocks + (int)blockIdx.x) * 32 + (int)(threadIdx.x & 31);
+    constexpr int stride = kCgBlocks * kCgThreads;
+    const bool any = (tid & ~31) < n;
+    RowLoop<W> rows(tid, n, sw, rlen, scol, sval, diag);
+    __syncwarp();
+    cluster_wait();   // every block's shared memory can be written
+    pdl_wait();
+    const bool first = sc->iters == 0;
+    const int mode = first ? kRho0 : zold ? kRZFlex : kRZ;
+    if (threadIdx.x == 0) S = *sc;
+    double a = 0.0, b = 0.0;
+#pragma unroll 4
+    for (int i = tid; i < n; i += stride) {
+        const double ri = r[i], zi = z[i];
+        a = fmad(ri, zi, a);
+        if (mode == kRZFlex) b = fmad(ri, zi - zold[i], b);
+    }
+    a = cluster_sum(a, any, sh, slot[0]);
+    if (mode == kRZFlex) b = cluster_sum(b, any, sh, slot[1]);
+    if (threadIdx.x == 0) cg_scalars(mode, a, b, &S, nullptr);
+    __syncthreads();
+    const double beta = S.beta;
+#pragma unroll 4
+    for (int i = tid; i < n; i += stride) {
+        const double zi = z[i];
+        p[i] = first ? zi : zi + beta * p[i];
+        if (zold) zold[i] = zi;
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();   // p is complete
+    double acc = 0.0, pi = 0.0;
+    rows.template run<false>(
+        FromL2{p}, &sc->status,
+        [&](int row, double d) {
+            pi = p[row];
+            return d * pi;
+        },
+        [&](int row, double v) {
+            q[row] = v;
+            acc = fmad(pi, v, acc);
+        });
+    acc = cluster_sum(acc, any, sh, slot[2]);
+    if (threadIdx.x == 0) cg_scalars(kPQ, acc, 0.0, &S, nullptr);
+    __syncthreads();
+    const double alpha = S.alpha;
+    double rr = 0.0;
+#pragma unroll 4
+    for (int i = tid; i < n; i += stride) {
+        x[i] += alpha * p[i];
+        const double v = r[i] - alpha * q[i];
+        r[i] = v;
+        rr = fmad(v, v, rr);
+    }
+    rr = cluster_sum(rr, any, sh, slot[3]);
+    if (cluster_rank() != 0 || threadIdx.x != 0) return;
+    cg_scalars(kRR, rr, 0.0, &S, nullptr);
+    sc->rr = S.rr;
+    sc->rho = S.rho;
+    sc->pq = S.pq;
+    sc->alpha = S.alpha;
+    sc->beta = S.beta;
+    sc->done = S.done;
+    sc->iters = S.iters;
+    if (S.status != 0) sc->status = S.status;   // an index out of range may have set it meanwhile
+    cg_continue(cond, sc);
+}
+
 // ---------------------------------------------------------------------------
 // BiCGSTAB (level 0, float64, smoothing order) with its scalars on the device.
 // Each kernel that ends in dot products combines them with the deterministic
@@ -1843,7 +1971,8 @@ __global__ void __launch_bounds__(kBlock) k_cg_p(int n, const double* __restrict
 // ---------------------------------------------------------------------------
 enum BiMode : int { kBiStart = 0, kBiRtv = 1, kBiHalf = 2, kBiW = 3, kBiUpdate = 4 };
 
-__device__ void finish_bi(double v0, double v1, double* partials, double* partials2,
+// true in the thread that applied the scalar step
+__device__ bool finish_bi(double v0, double v1, double* partials, double* partials2,
                           unsigned int* counter, BiScalars* bs, int mode, double* sh) {
     __shared__ bool last;
     if (threadIdx.x == 0) {
@@ -1854,7 +1983,7 @@ __device__ void finish_bi(double v0, double v1, double* partials, double* partia
         last = (t == gridDim.x - 1);
     }
     __syncthreads();
-    if (!last) return;
+    if (!last) return false;
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
         a += __ldcg(partials + i);
@@ -1862,7 +1991,7 @@ __device__ void finish_bi(double v0, double v1, double* partials, double* partia
     }
     a = block_sum(a, sh);
     b = block_sum(b, sh);
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0) return false;
     *counter = 0u;
     // a NaN or infinity in a dot product of the iteration ends the solve
     if (!finite_dot(a) || !finite_dot(b)) {
@@ -1873,7 +2002,7 @@ __device__ void finish_bi(double v0, double v1, double* partials, double* partia
         }
         bs->status = AMG_ENONFINITE;
         bs->why = 4;
-        return;
+        return true;
     }
     switch (mode) {
         case kBiStart:   // a = r.r
@@ -1926,6 +2055,7 @@ __device__ void finish_bi(double v0, double v1, double* partials, double* partia
             bs->done = !(bs->rel > bs->tol);
             break;
     }
+    return true;
 }
 
 // r = b - A x, rt = r, and the start scalars from r.r
@@ -1940,7 +2070,7 @@ __global__ void __launch_bounds__(kBlock) k_bi_start(int n, int64_t sw,
                                                      unsigned int* counter, BiScalars* bs) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
-    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
+    RowLoop<W> rows(blockIdx.x * blockDim.x + threadIdx.x, n, sw, rlen, scol, sval, diag);
     pdl_wait();
     double a = 0.0;
     rows.template run<true>(
@@ -1981,7 +2111,7 @@ __global__ void __launch_bounds__(kBlock) k_bi_spmv(int n, int64_t sw,
                                                     unsigned int* counter, BiScalars* bs, int mode) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
-    RowLoop<W> rows(n, sw, rlen, scol, sval, diag);
+    RowLoop<W> rows(blockIdx.x * blockDim.x + threadIdx.x, n, sw, rlen, scol, sval, diag);
     pdl_wait();
     if (bs->status || (mode == kBiW && bs->half)) return;
     double a = 0.0, b = 0.0;
@@ -2017,22 +2147,39 @@ __global__ void __launch_bounds__(kBlock) k_bi_half(int n, const double* r, cons
     finish_bi(ta, 0.0, partials, partials2, counter, bs, kBiHalf, sh);
 }
 
+// Condition of the BiCGSTAB loop (a WHILE graph node), evaluated before every
+// iteration: stop once converged or broken down, at maxit, or when
+// rho = rt.r is zero (a breakdown); the evaluation count is a second bound.
+__device__ __forceinline__ void bi_loop(const LoopCond& cond, BiScalars* bs) {
+    if (!cond.on) return;
+    const int32_t loops = ++bs->loops;
+    const int go = bi_continue(*bs) && loops <= bs->maxit + 1;
+    cudaGraphSetConditional(cond.h, go ? 1u : 0u);
+}
+
 // x += alpha y + w z, r = s - w t, r.r and rt.r; after a converged half step
 // only x += alpha y
 __global__ void __launch_bounds__(kBlock) k_bi_update(int n, double* x, const double* y,
                                                       const double* z, const double* s,
                                                       const double* t, double* r, const double* rt,
                                                       double* partials, double* partials2,
-                                                      unsigned int* counter, BiScalars* bs) {
+                                                      unsigned int* counter, BiScalars* bs,
+                                                      const LoopCond cond) {
     __shared__ double sh[kBlock / 32];
     pdl_launch_dependents();
     pdl_wait();
-    if (bs->status) return;
+    // stopped already (a converged half step is done): the loop ends here
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (bs->status) {
+        if (first) bi_loop(cond, bs);
+        return;
+    }
     const double alpha = bs->alpha;
     const int stride = gridDim.x * blockDim.x;
     if (bs->half) {
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
             x[i] = fmad(alpha, y[i], x[i]);
+        if (first) bi_loop(cond, bs);
         return;
     }
     const double w = bs->w;
@@ -2046,17 +2193,11 @@ __global__ void __launch_bounds__(kBlock) k_bi_update(int n, double* x, const do
     }
     const double ta = block_sum(a, sh);
     const double tb = block_sum(b, sh);
-    finish_bi(ta, tb, partials, partials2, counter, bs, kBiUpdate, sh);
+    if (finish_bi(ta, tb, partials, partials2, counter, bs, kBiUpdate, sh)) bi_loop(cond, bs);
 }
 
-// Condition of the BiCGSTAB loop (a WHILE graph node), evaluated before every
-// iteration: stop once converged or broken down, at maxit, or when
-// rho = rt.r is zero (a breakdown); the evaluation count is a second bound.
-__global__ void k_bi_continue(cudaGraphConditionalHandle h, BiScalars* bs) {
-    const int32_t loops = ++bs->loops;
-    const int go = bi_continue(*bs) && loops <= bs->maxit + 1;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
-}
+// The condition before the first iteration.
+__global__ void k_bi_continue(const LoopCond cond, BiScalars* bs) { bi_loop(cond, bs); }
 
 inline int blocks_for(int64_t threads) { return (int)((threads + kBlock - 1) / kBlock); }
 
@@ -2586,11 +2727,6 @@ void launch_vrecords(const VRec* const* recs, int n, cudaStream_t s) {
     }
 }
 
-void launch_cg_continue(cudaGraphConditionalHandle h, PcgScalars* sc, cudaStream_t s) {
-    k_cg_continue<<<1, 1, 0, s>>>(h, sc);
-    AMG_CUDA_TRY(cudaGetLastError());
-}
-
 void launch_dense_gemv_f32(int n, int ld, const float* M, const float* b, float* x, cudaStream_t s) {
     if ((reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(M)) & 15 || ld % 4 || ld < n)
         throw Error{AMG_EINVAL, "float32 coarsest solve: operands must be 16-byte aligned"};
@@ -2668,9 +2804,58 @@ void wait_selftest(long long limit, cudaStream_t s, int32_t* status, double* ela
 }
 
 void launch_cg_update(int n, double* x, double* r, const double* p, const double* q, CgWork& w,
-                      cudaStream_t s) {
+                      LoopCond cond, cudaStream_t s) {
     launch_kernel(k_cg_update, reduction_blocks(n), kBlock, 0, s, n, x, r, p, q, w.partials, w.counters + 2,
-                                                       w.sc);
+                                                       w.sc, cond);
+}
+
+namespace {
+
+template <int W>
+cudaLaunchConfig_t cg_cluster_config(cudaLaunchAttribute* attr, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCgBlocks);
+    cfg.blockDim = dim3(kCgThreads);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kCgBlocks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    AMG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_cg_cluster<W>),
+                                      cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    return cfg;
+}
+
+}  // namespace
+
+bool cg_cluster_fits(const DevLevel& L) {
+    if (L.n > kCgClusterRows) return false;
+    int clusters = 0;
+    cudaLaunchAttribute attr[2];
+    cudaError_t e = cudaSuccess;
+    AMG_WIDTH_DISPATCH(L.width, {
+        const cudaLaunchConfig_t cfg = cg_cluster_config<W>(attr, nullptr);
+        e = cudaOccupancyMaxActiveClusters(&clusters, k_cg_cluster<W>, &cfg);
+    });
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && clusters > 0;
+}
+
+void launch_cg_cluster(const DevLevel& L, double* r, const double* z, double* zold, double* p, double* q,
+                       double* x, CgWork& w, LoopCond cond, cudaStream_t s) {
+    AMG_WIDTH_DISPATCH(L.width, {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = cg_cluster_config<W>(attr, s);
+        if (t_launch_overlap) {
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
+            cfg.numAttrs = 2;
+        }
+        AMG_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_cg_cluster<W>, L.n, L.sw, (const uint16_t*)L.rlen,
+                                        (const int32_t*)L.scol, (const double*)L.sval, (const double*)L.diag,
+                                        r, z, zold, p, q, x, w.sc, cond));
+    });
 }
 
 void launch_cg_rz(int n, const double* r, const double* z, const double* zold, double* p,
@@ -2712,13 +2897,13 @@ void launch_bi_half(int n, const double* r, const double* v, double* sv, CgWork&
 
 void launch_bi_update(int n, double* x, const double* y, const double* z, const double* sv,
                       const double* t, double* r, const double* rt, CgWork& wk, BiScalars* bs,
-                      cudaStream_t s) {
+                      LoopCond cond, cudaStream_t s) {
     launch_kernel(k_bi_update, reduction_blocks(n), kBlock, 0, s, n, x, y, z, sv, t, r, rt,
-                  wk.partials, wk.partials2, wk.counters + 8, bs);
+                  wk.partials, wk.partials2, wk.counters + 8, bs, cond);
 }
 
-void launch_bi_continue(cudaGraphConditionalHandle h, BiScalars* bs, cudaStream_t s) {
-    k_bi_continue<<<1, 1, 0, s>>>(h, bs);
+void launch_bi_continue(LoopCond cond, BiScalars* bs, cudaStream_t s) {
+    k_bi_continue<<<1, 1, 0, s>>>(cond, bs);
     AMG_CUDA_TRY(cudaGetLastError());
 }
 

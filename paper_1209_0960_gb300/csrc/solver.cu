@@ -936,9 +936,7 @@ void apply_shapes(amg_ctx* c) {
 // preconditioned CG on level-0 vectors in smoothing order (c->bb, c->x)
 // ---------------------------------------------------------------------------
 
-// One CG iteration is two parts.  A: q = A p, alpha, x/r update, copy of the
-// CG scalars to the host.  B: z = B r, beta, p update.
-void cg_part_a(amg_ctx* c, bool copy_back = true) {
+void cg_spmv_update(amg_ctx* c, LoopCond cond) {
     DevLevel& L0 = c->dl[0];
     const int n = L0.n;
     cudaStream_t s = c->stream;
@@ -946,26 +944,49 @@ void cg_part_a(amg_ctx* c, bool copy_back = true) {
         ProfScope ps(c, kKCgSpmv, (double)L0.nnz_off * 12 + 2.0 * n + 24.0 * n);
         launch_cg_spmv_pq(L0, c->pv, c->q, c->work, s);
     }
+    ProfScope ps(c, kKCgUpdate, 48.0 * n);
+    launch_cg_update(n, c->x, c->r, c->pv, c->q, c->work, cond, s);
+}
+
+// beta and p from z = B r (first: rho and p = z)
+void cg_direction(amg_ctx* c, bool first) {
+    if (c->cg_cluster) return;   // in part A
+    const int n = c->dl[0].n;
+    cudaStream_t s = c->stream;
+    if (first) {
+        launch_cg_rz(n, c->r, c->z, nullptr, c->pv, c->work, kRho0, s);
+        if (c->flexible)
+            AMG_CUDA_TRY(cudaMemcpyAsync(c->zold, c->z, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        return;
+    }
     {
-        ProfScope ps(c, kKCgUpdate, 48.0 * n);
-        launch_cg_update(n, c->x, c->r, c->pv, c->q, c->work, s);
+        ProfScope ps(c, kKCgDot, (c->flexible ? 24.0 : 16.0) * n);
+        launch_cg_rz(n, c->r, c->z, c->zold, c->pv, c->work, c->flexible ? kRZFlex : kRZ, s);
+    }
+    ProfScope ps(c, kKCgP, (c->flexible ? 32.0 : 24.0) * n);
+    launch_cg_p(n, c->z, c->pv, c->flexible ? c->zold : nullptr, c->work, s);
+}
+
+// One CG iteration is two parts.  A: q = A p, alpha, x/r update, copy of the
+// CG scalars to the host.  B: z = B r, beta, p update.  On small systems all but
+// z = B r is one launch of part A.
+void cg_part_a(amg_ctx* c, bool copy_back = true, LoopCond cond = {}) {
+    DevLevel& L0 = c->dl[0];
+    const int n = L0.n;
+    cudaStream_t s = c->stream;
+    if (c->cg_cluster) {
+        ProfScope ps(c, kKCgSpmv, (double)L0.nnz_off * 12 + (c->flexible ? 130.0 : 114.0) * n);
+        launch_cg_cluster(L0, c->r, c->z, c->flexible ? c->zold : nullptr, c->pv, c->q, c->x, c->work, cond, s);
+    } else {
+        cg_spmv_update(c, cond);
     }
     if (copy_back)
         AMG_CUDA_TRY(cudaMemcpyAsync(c->sc_host, c->work.sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost, s));
 }
 
 void cg_part_b(amg_ctx* c) {
-    const int n = c->dl[0].n;
-    cudaStream_t s = c->stream;
     precondition(c, c->r, c->z);
-    {
-        ProfScope ps(c, kKCgDot, (c->flexible ? 24.0 : 16.0) * n);
-        launch_cg_rz(n, c->r, c->z, c->zold, c->pv, c->work, c->flexible ? kRZFlex : kRZ, s);
-    }
-    {
-        ProfScope ps(c, kKCgP, (c->flexible ? 32.0 : 24.0) * n);
-        launch_cg_p(n, c->z, c->pv, c->flexible ? c->zold : nullptr, c->work, s);
-    }
+    cg_direction(c, false);
 }
 
 bool cg_graphs(const amg_ctx* c) { return c->use_graphs && !c->prof.on; }
@@ -1001,12 +1022,8 @@ void cg_start(amg_ctx* c, double tol, int32_t maxit) {
 
 // first preconditioning: z = B r, rho = r.z, p = z
 void cg_first_direction(amg_ctx* c) {
-    const int n = c->dl[0].n;
-    cudaStream_t s = c->stream;
     precondition(c, c->r, c->z);
-    launch_cg_rz(n, c->r, c->z, nullptr, c->pv, c->work, kRho0, s);
-    if (c->flexible)
-        AMG_CUDA_TRY(cudaMemcpyAsync(c->zold, c->z, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+    cg_direction(c, true);
 }
 
 // true residual of the final iterate into c->norm_dev
@@ -1023,14 +1040,13 @@ void cg_fill_info(const amg_ctx* c, int status, double rr_true, amg_solve_info* 
     info->device_loop = c->last_device_loop;
 }
 
-// A Krylov iteration loop as one graph: `pre` on the context stream, then
-// `cond(h, stream)` (a one-thread kernel setting the loop condition h from the
-// device scalars), then a WHILE node whose body is `body` followed by `cond`
-// again, then `post`.  No iteration waits on the host; the scalars come back
-// once, in `post`.  Returns nullptr (and clears the error) when the runtime
-// refuses the graph.
-template <typename Pre, typename Cond, typename Body, typename Post>
-cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Cond&& cond, Body&& body, Post&& post) {
+// A Krylov iteration loop as one graph: `pre(h)` on the context stream, then a
+// WHILE node whose body is `body(h)`, then `post`.  The last kernel of pre and
+// of body sets the loop condition h from the device scalars.  No iteration waits
+// on the host; the scalars come back once, in `post`.  Returns nullptr (and
+// clears the error) when the runtime refuses the graph.
+template <typename Pre, typename Body, typename Post>
+cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Body&& body, Post&& post) {
     if (!c->stream_body)
         AMG_CUDA_TRY(cudaStreamCreateWithFlags(&c->stream_body, cudaStreamNonBlocking));
     cudaStream_t s = c->stream;
@@ -1053,7 +1069,6 @@ cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Cond&& cond, Body&& bod
         return nullptr;
     }
     try {
-        pre();
         cudaStreamCaptureStatus st;
         cudaGraph_t cg = nullptr;
         const cudaGraphNode_t* deps = nullptr;
@@ -1063,7 +1078,7 @@ cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Cond&& cond, Body&& bod
         cudaError_t e = cudaStreamGetCaptureInfo(s, &st, nullptr, &cg, &deps, &edges, &nd);
         if (ok(e)) e = cudaGraphConditionalHandleCreate(&h, cg, 0, cudaGraphCondAssignDefault);
         if (!ok(e)) { fail(e); return nullptr; }
-        cond(h, s);
+        pre(h);
         e = cudaStreamGetCaptureInfo(s, &st, nullptr, &cg, &deps, &edges, &nd);
         cudaGraphNodeParams prm = {};
         prm.type = cudaGraphNodeTypeConditional;
@@ -1078,8 +1093,7 @@ cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Cond&& cond, Body&& bod
         if (!ok(e)) { fail(e); return nullptr; }
         body_capturing = true;
         c->stream = c->stream_body;
-        body();
-        cond(h, c->stream);
+        body(h);
         c->stream = s;
         cudaGraph_t bg = nullptr;
         e = cudaStreamEndCapture(c->stream_body, &bg);
@@ -1111,19 +1125,18 @@ cudaGraphExec_t build_while_graph(amg_ctx* c, Pre&& pre, Cond&& cond, Body&& bod
 // The iteration loop of PCG as one graph: the first direction (z = B r,
 // rho, p = z) and the first update (q = A p, alpha, x, r, ||r||), then a
 // WHILE node whose body is one more iteration (z = B r, beta, p; q = A p,
-// alpha, x, r, ||r||).  The loop condition kernel runs after each update.
+// alpha, x, r, ||r||).  The update's last block sets the loop condition.
 // The launches are those of the host-driven loop, in the same order.
 cudaGraphExec_t build_solve_graph(amg_ctx* c) {
     return build_while_graph(
         c,
-        [&] {
+        [&](cudaGraphConditionalHandle h) {
             cg_first_direction(c);
-            cg_part_a(c, false);
+            cg_part_a(c, false, LoopCond{h, 1});
         },
-        [&](cudaGraphConditionalHandle h, cudaStream_t st) { launch_cg_continue(h, c->work.sc, st); },
-        [&] {
+        [&](cudaGraphConditionalHandle h) {
             cg_part_b(c);
-            cg_part_a(c, false);
+            cg_part_a(c, false, LoopCond{h, 1});
         },
         [&] {
             AMG_CUDA_TRY(cudaMemcpyAsync(c->sc_host, c->work.sc, sizeof(PcgScalars),
@@ -1222,7 +1235,7 @@ int pcg(amg_ctx* c, double tol, int32_t maxit, amg_solve_info* info) {
 // with a device-side WHILE node; the host-driven loop (profiling, or a
 // refused graph) reads the scalars back once per iteration.
 // ---------------------------------------------------------------------------
-void bi_iteration(amg_ctx* c) {
+void bi_iteration(amg_ctx* c, LoopCond cond = {}) {
     DevLevel& L0 = c->dl[0];
     const int n = L0.n;
     cudaStream_t s = c->stream;
@@ -1237,7 +1250,7 @@ void bi_iteration(amg_ctx* c) {
     // after a converged half step this V-cycle's result is not used
     precondition(c, c->bs, z);
     launch_bi_spmv(L0, z, c->bt, c->bs, true, c->work, c->bsc, c->stream);
-    launch_bi_update(n, x, c->by, z, c->bs, c->bt, r, c->rt, c->work, c->bsc, c->stream);
+    launch_bi_update(n, x, c->by, z, c->bs, c->bt, r, c->rt, c->work, c->bsc, cond, c->stream);
 }
 
 cudaGraphExec_t bicgstab_graph(amg_ctx* c) {
@@ -1247,9 +1260,8 @@ cudaGraphExec_t bicgstab_graph(amg_ctx* c) {
     if (state == 0) {
         auto build = [&] {
             return build_while_graph(
-                c, [] {},
-                [&](cudaGraphConditionalHandle h, cudaStream_t st) { launch_bi_continue(h, c->bsc, st); },
-                [&] { bi_iteration(c); },
+                c, [&](cudaGraphConditionalHandle h) { launch_bi_continue(LoopCond{h, 1}, c->bsc, c->stream); },
+                [&](cudaGraphConditionalHandle h) { bi_iteration(c, LoopCond{h, 1}); },
                 [&] {
                     AMG_CUDA_TRY(cudaMemcpyAsync(c->bsc_host, c->bsc, sizeof(BiScalars),
                                                  cudaMemcpyDeviceToHost, c->stream));
@@ -1520,18 +1532,9 @@ int pcg_async_poll(amg_ctx* c, bool* first) {
 void pcg_async_resume(amg_ctx* c, bool first) {
     AsyncCg& a = c->acg;
     t_launch_overlap = c->p.launch_overlap != 0;
-    const int n = c->dl[0].n;
-    cudaStream_t s = c->stream;
-    if (first) {
-        launch_cg_rz(n, c->r, c->z, nullptr, c->pv, c->work, kRho0, s);
-        if (c->flexible)
-            AMG_CUDA_TRY(cudaMemcpyAsync(c->zold, c->z, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    } else {
-        launch_cg_rz(n, c->r, c->z, c->zold, c->pv, c->work, c->flexible ? kRZFlex : kRZ, s);
-        launch_cg_p(n, c->z, c->pv, c->flexible ? c->zold : nullptr, c->work, s);
-    }
+    cg_direction(c, first);
     run_part_a(c);
-    AMG_CUDA_TRY(cudaEventRecord(a.ev, s));
+    AMG_CUDA_TRY(cudaEventRecord(a.ev, c->stream));
     a.state = AsyncCg::kIterating;
     AMG_CUDA_TRY(cudaGetLastError());
 }
@@ -1866,6 +1869,7 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     AMG_CUDA_TRY(cudaEventCreate(&c->ev1));
     AMG_CUDA_TRY(cudaStreamSynchronize(s));
 
+    c->cg_cluster = cg_cluster_fits(c->dl[0]);
     c->flexible = prm->flexible_cg > 0 ? 1 : 0;
     c->precision = prm->precision;
     if (c->precision == AMG_FP32_IN_FP64) ensure_fp32(c.get());
