@@ -26,7 +26,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["kernels.cu", "tail.cu", "setup_device.cu", "solver.cu", "noalloc.cu", "server.cu",
               "aggregate_device.cu"]
 CPP_SOURCES = ["host_setup.cpp"]
-HEADERS = ["device.h", "device_util.cuh", "host_setup.h"]
+HEADERS = ["device.h", "device_util.cuh", "host_setup.h", "row_tiles.h"]
 
 
 def _deps():

@@ -35,6 +35,7 @@
 
 #include "device.h"
 #include "device_util.cuh"
+#include "row_tiles.h"
 
 namespace amg {
 
@@ -100,9 +101,7 @@ int device_of_pointer(const void* p, const char* name) {
 // adds its squares over all its rows before one reduction per block at the end.
 // Every row is still b_i - A_i0 x_0 - ... in stored order.
 //
-// Rows are read in tiles of kNaTile entries per warp (32 rows of a 7-point
-// stencil fit in one); longer runs take more tiles.
-constexpr int kNaTile = 224;
+// Rows are read in tiles of kNaTile entries per warp (row_tiles.h).
 constexpr int kNaWarps = kNaBlock / 32;
 
 __device__ __forceinline__ void copy_async8(void* dst, const void* src) {
@@ -161,15 +160,15 @@ __global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm(
         copy_wait<1>();
         __syncwarp();
         int k = max(k0, s);   // (never left of the tile, also for a malformed row_ptr)
-        for (int base = s;;) {
-            const int end = min(k1, base + kNaTile);
+        RowTiles tile(s, e);
+        for (;;) {
+            const int base = tile.base, end = tile.end_in_tile(k1);
 #pragma unroll 4
             for (; k < end; ++k)
                 t = __fma_rn(-sv[warp][buf][k - base], x[sc[warp][buf][k - base]], t);
-            base += kNaTile;
-            if (base >= e) break;
+            if (!tile.next()) break;
             __syncwarp();
-            fetch(buf, base, e);
+            fetch(buf, tile.base, e);
             copy_commit();
             copy_wait<0>();
             __syncwarp();
