@@ -10,13 +10,14 @@
 // allocation: the per-block partial sums of its deterministic two-stage
 // reduction live in a fixed file-scope device array.
 //
-// The array holds kMaxBlocks partial sums.  Matrices of up to kMaxBlocks * 256 =
-// 16,777,216 rows are accepted and larger ones are rejected with AMG_EINVAL.  Every GPU that loads the library holds the array
-// (512 KiB plus a counter) until the process exits.  All calls share it and it
-// keeps the last call's contents; each call clears the arrival counter before
-// its kernel runs.  Calls that overlap on the GPU (concurrent streams, or
-// several host threads) race on the array and must be serialised by the
-// caller.
+// The array holds kMaxBlocks partial sums, one per 256 rows where a thread takes
+// a row (the other kernel has at most five blocks per SM), so matrices of up to
+// kMaxBlocks * 256 = 16,777,216 rows are accepted and larger ones are rejected
+// with AMG_EINVAL.  Every GPU that loads the library holds the array (512 KiB
+// plus a counter) until the process exits.  All calls share it and it keeps the
+// last call's contents; each call clears the arrival counter before its kernel
+// runs.  Calls that overlap on the GPU (concurrent streams, or several host
+// threads) race on the array and must be serialised by the caller.
 //
 // Set-up: the first call on each device looks up the array's device address
 // with cudaGetSymbolAddress while that device is current, and caches it for
@@ -89,21 +90,56 @@ int device_of_pointer(const void* p, const char* name) {
     return at.device;
 }
 
+constexpr int kNaWarps = kNaBlock / 32;
+
+// The sum of v over all threads: per block in a fixed order, then the last block
+// to finish adds the block sums in index order and writes the square root.
+__device__ __forceinline__ void finish_norm(double v, NoAllocScratch* __restrict__ scratch,
+                                            double* __restrict__ out) {
+    __shared__ double sh[kNaWarps];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane == 0) sh[warp] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double q = 0.0;
+        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
+        scratch->partial[blockIdx.x] = q;
+        __threadfence();
+        last = atomicAdd(&scratch->counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    double a = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kNaBlock) a += __ldcg(scratch->partial + i);
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    __syncthreads();
+    if (lane == 0) sh[warp] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double q = 0.0;
+        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
+        *out = sqrt(q);
+        scratch->counter = 0u;
+    }
+}
+
 // ||b - A x||^2 over the rows, a warp per 32 consecutive rows at a time.
 //
 // One thread per row reading its CSR row directly touches a different line per
 // lane and entry, and summing the squares of every 32 rows costs five warp-wide
 // float64 additions where the rows themselves cost eight: on GB300, whose
 // float64 pipe takes about as long for this kernel as HBM does, that was half
-// the copy rate (95 us for 3.0M rows, 312 MB; now 79 us).  Here the entries of a warp's 32
-// rows, which are contiguous, are copied line by line into shared memory with
-// cp.async, the next 32 rows' while the current ones are summed, and each thread
-// adds its squares over all its rows before one reduction per block at the end.
+// the copy rate (97 us for 3.0M rows, 312 MB; now 81 us).  Here the entries of a
+// warp's 32 rows, which are contiguous, are copied line by line into shared memory
+// with cp.async, the next 32 rows' while the current ones are summed, and each
+// thread adds its squares over all its rows before one reduction per block at the
+// end.
 // Every row is still b_i - A_i0 x_0 - ... in stored order.
 //
-// Rows are read in tiles of kNaTile entries per warp (row_tiles.h).
-constexpr int kNaWarps = kNaBlock / 32;
-
+// Rows are read in tiles of kNaTile entries per warp (row_tiles.h): 32 rows of a
+// 7-point stencil.
 __device__ __forceinline__ void copy_async8(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -122,8 +158,6 @@ __global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm(
     NoAllocScratch* __restrict__ scratch, double* __restrict__ out) {
     __shared__ double sv[kNaWarps][2][kNaTile];
     __shared__ int32_t sc[kNaWarps][2][kNaTile];
-    __shared__ double sh[kNaWarps];
-    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int groups = (n + 31) >> 5, stride = (int)gridDim.x * kNaWarps;
     const int g0 = (int)blockIdx.x * kNaWarps + warp;
@@ -177,31 +211,31 @@ __global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm(
         __syncwarp();   // the buffer is filled again in the next round
         k0 = k0n, k1 = k1n, k0n = k0f, k1n = k1f, s = sn, e = en;
     }
-    double v = acc;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double q = 0.0;
-        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
-        scratch->partial[blockIdx.x] = q;
-        __threadfence();
-        last = atomicAdd(&scratch->counter, 1u) == gridDim.x - 1;
+    finish_norm(acc, scratch, out);
+}
+
+// The same norm with one thread per row reading its CSR row directly: rows of
+// more than kNaTile / 32 entries on the mean.  There a tile holds the rows of a
+// few lanes only, the float64 pipe takes a warp's instruction at the same rate
+// however few of its lanes are active, and the tiles after a group's first are
+// waited for.  A longer row also uses more of each line it touches.  Tiled
+// kernel against this one (GB300): 27 entries a row, 2.1M rows 415 against 232 us
+// and 262k rows 66 against 38; 12.5 a row, 300k rows 34.5 against 29; 9 a row, 1M
+// rows 53 against 47; the other way round 7 a row, 3.0M rows 81 against 97; 5 a
+// row, 1M rows 26 against 37; 3 a row, 3M rows 48 against 75; rows of uneven
+// length, 5.9 a row on the mean, 300k rows 20.7 against 21.8.
+__global__ void __launch_bounds__(kNaBlock) k_csr_residual_norm_rows(
+    int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+    const double* __restrict__ va, const double* __restrict__ b, const double* __restrict__ x,
+    NoAllocScratch* __restrict__ scratch, double* __restrict__ out) {
+    const int row = blockIdx.x * kNaBlock + threadIdx.x;
+    double v = 0.0;
+    if (row < n) {
+        double t = b[row];
+        for (int k = rp[row]; k < rp[row + 1]; ++k) t = __fma_rn(-va[k], x[ci[k]], t);
+        v = t * t;
     }
-    __syncthreads();
-    if (!last) return;
-    double a = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += kNaBlock) a += __ldcg(scratch->partial + i);
-    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-    __syncthreads();
-    if (lane == 0) sh[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double q = 0.0;
-        for (int w = 0; w < kNaWarps; ++w) q += sh[w];
-        *out = sqrt(q);
-        scratch->counter = 0u;
-    }
+    finish_norm(v, scratch, out);
 }
 
 }  // namespace
@@ -234,13 +268,19 @@ extern "C" int amg_residual_norm_noalloc(const amg_csr* A, const double* b_dev,
         NoAllocScratch* scratch = scratch_for_current_device();
         cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
         AMG_CUDA_TRY(cudaMemsetAsync(&scratch->counter, 0, sizeof(unsigned int), s));
-        // as many blocks as are resident at once (five per SM by their shared
-        // memory), each taking every grid-th 256 rows
-        int sms = 0;
-        AMG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int grid = std::min((A->n + kNaBlock - 1) / kNaBlock, std::max(1, std::min(5 * sms, kMaxBlocks)));
-        k_csr_residual_norm<<<grid, kNaBlock, 0, s>>>(A->n, A->row_ptr, A->col, A->val, b_dev, x_dev,
-                                                      scratch, norm_dev);
+        const int blocks = (A->n + kNaBlock - 1) / kNaBlock;   // at most kMaxBlocks
+        if ((int64_t)A->nnz * 32 > (int64_t)A->n * kNaTile) {
+            k_csr_residual_norm_rows<<<blocks, kNaBlock, 0, s>>>(A->n, A->row_ptr, A->col, A->val, b_dev,
+                                                                 x_dev, scratch, norm_dev);
+        } else {
+            // as many blocks as are resident at once (five per SM by their
+            // shared memory), each taking every grid-th 256 rows
+            int sms = 0;
+            AMG_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+            const int grid = std::min(blocks, std::max(1, 5 * sms));
+            k_csr_residual_norm<<<grid, kNaBlock, 0, s>>>(A->n, A->row_ptr, A->col, A->val, b_dev, x_dev,
+                                                          scratch, norm_dev);
+        }
         AMG_CUDA_TRY(cudaGetLastError());
         set_last_error("");
         return AMG_OK;

@@ -1,6 +1,7 @@
 """The allocation-free residual norm on rows of any length: groups of 32 rows
-with no entry, one, a full tile of 224, one more, and several thousand, in
-matrices whose last group is short, against numpy."""
+with no entry, one, a full tile of 224, one more (the limit between its two
+kernels), and several thousand, in matrices whose last group is short, against
+numpy."""
 
 import numpy as np
 import pytest
@@ -19,6 +20,10 @@ def _lengths(kind, n, rng):
         return np.zeros(n, dtype=np.int64)
     if kind == "mixed":   # some rows empty, some of thousands of entries
         return rng.choice([0, 1, 7, 27, 300, 5000], size=n, p=[0.2, 0.2, 0.3, 0.2, 0.08, 0.02])
+    if kind == "few long":   # short on the mean: several tiles in some groups
+        out = rng.integers(0, 4, size=n)
+        out[rng.integers(0, n, size=1 + n // 4000)] += 3000
+        return out
     out = np.zeros(n, dtype=np.int64)   # groups of `kind` entries, spread over their rows
     for g in range(0, n, 32):
         m = min(32, n - g)
@@ -27,7 +32,7 @@ def _lengths(kind, n, rng):
 
 
 @pytest.mark.parametrize("n", [1, 31, 33, 8191, 60_013])
-@pytest.mark.parametrize("kind", ["empty", 1, 224, 225, 449, 864, "mixed"])
+@pytest.mark.parametrize("kind", ["empty", 1, 224, 225, 449, 864, "mixed", "few long"])
 def test_rows_of_any_length(kind, n):
     rng = np.random.default_rng(n)
     lens = _lengths(kind, n, rng)
