@@ -396,14 +396,19 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
             const TailLevel<T>& L = lev[l];
             const int C = L.ncolours;
             const T* e = xs + lev[l + 1].xoff;
-            // x += omega P e on the own rows of colour >= 1
-            for (int i = blk[L.blk0 + 1].lo + slot; i < L.nown; i += kPer) {
-                const int oi = L.own0 + i;
-                const OwnRow o = orow[oi];
+            // x += omega P e on the own rows of colour >= 1.  All lanes of a row
+            // read its x; lane 0 replaces it once they have (the other lanes
+            // send the sum to the blocks that read the row).
+            for (int k0 = blk[L.blk0 + 1].lo; warp_has(L.nown, k0); k0 += kPer) {
+                const int oi = L.own0 + k0 + slot;
+                OwnRow o = {0xffff, 0, 0, 0, 0u, 0u};
+                if (k0 + slot < L.nown) o = orow[oi];
                 const int g = o.row != 0xffff ? oagg[oi] : 0xffff;
-                if (g == 0xffff || !index_ok(g, L.nc, err)) continue;
-                const T w = kScaled ? omega * oaggw[oi] : omega;
-                publish(o, L.xoff + o.row, fmad(w, e[g], xs[L.xoff + o.row]));
+                const bool has = g != 0xffff && index_ok(g, L.nc, err);
+                T v = T(0);
+                if (has) v = fmad(kScaled ? omega * oaggw[oi] : omega, e[g], xs[L.xoff + o.row]);
+                __syncwarp();
+                if (has) publish(o, L.xoff + o.row, v);
             }
             __syncwarp();
             tail_sync<NC>();
