@@ -49,11 +49,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 
 // thread-block clusters: the barrier in its two halves (release, acquire), the
-// block's rank, and stores into another block's shared memory
+// block's rank, and stores into another block's shared memory.  The barrier's
+// aligned forms want the whole warp at the same instruction, which the compiler
+// does not know: the warp meets here, whatever the caller's loops did.
 __device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -1855,7 +1855,6 @@ __device__ __forceinline__ double cluster_sum(double v, bool any, double* sh, do
         const double t = group_sum<32>(lane < kCgThreads / 32 ? sh[lane] : 0.0);
         if (lane < kCgBlocks) st_cluster(map_rank(smem_u32(slot + cluster_rank()), (uint32_t)lane), t);
     }
-    __syncwarp();
     cluster_arrive();
     cluster_wait();
     return warp == 0 ? group_sum<32>(lane < kCgBlocks ? slot[lane] : 0.0) : 0.0;
@@ -1895,7 +1894,6 @@ __global__ void __launch_bounds__(kCgThreads, 1)
     constexpr int stride = kCgBlocks * kCgThreads;
     const bool any = (tid & ~31) < n;
     RowLoop<W> rows(tid, n, sw, rlen, scol, sval, diag);
-    __syncwarp();
     cluster_wait();   // every block's shared memory can be written
     pdl_wait();
     const bool first = sc->iters == 0;
@@ -1919,7 +1917,6 @@ __global__ void __launch_bounds__(kCgThreads, 1)
         p[i] = first ? zi : zi + beta * p[i];
         if (zold) zold[i] = zi;
     }
-    __syncwarp();
     cluster_arrive();
     cluster_wait();   // p is complete
     double acc = 0.0, pi = 0.0;

@@ -238,7 +238,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
                 publish(o, L.xoff + o.row, sx * od[oi]);
             }
         }
-        __syncwarp();
         tail_sync<NC>();
     };
 
@@ -278,7 +277,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
                     const OwnRow o = orow[oi];
                     if (o.row != 0xffff) publish(o, L.xoff + o.row, ob[oi] * od[oi]);
                 }
-                __syncwarp();
                 tail_sync<NC>();
             }
 #pragma unroll 1
@@ -295,7 +293,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
                     const T s = sum(part(lead ? ob[oi] - os[oi] : T(0), o, false, L.n, x));
                     if (lead) L.r[o.row] = s;
                 }
-                __syncwarp();
                 tail_sync<NC>();
             }
             // right-hand side of the own rows of the next level
@@ -339,7 +336,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
                     }
                 }
             }
-            __syncwarp();
             if (coarsest) tail_sync<NC>();
             else __syncthreads();
         }
@@ -410,7 +406,6 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const TailBatch batch)
                 __syncwarp();
                 if (has) publish(o, L.xoff + o.row, v);
             }
-            __syncwarp();
             tail_sync<NC>();
 #pragma unroll 1
             for (int c = 0; c < C; ++c) pass(L, c, Both());
