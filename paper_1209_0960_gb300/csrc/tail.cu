@@ -108,6 +108,12 @@ struct TailDesc {
     int32_t* err;
 };
 
+// What an index outside its level becomes in an image: positions have 16 bits
+// there, and a cut one could fall inside the level again.  It is past the rows
+// of every level (kTailMaxRows), so the checked build's kernel reports it each
+// time it meets it, as the other kernels do.
+constexpr uint16_t kTailOut = 0xfffe;
+
 struct TailBatch {
     const void* desc[kMaxVBatch];
 };
@@ -469,9 +475,10 @@ __global__ void __launch_bounds__(kPackThreads) k_tail_pack(const TailDesc<T>* D
                 for (int t = 0; t < o.low + o.up; ++t) {
                     const int64_t e = base + 32 * (int64_t)(t < o.low ? t : L.last - (t - o.low));
                     const int j = L.scol[e];
-                    col[t] = (uint16_t)j;
+                    const bool in = index_ok(j, L.n, D.err);
+                    col[t] = in ? (uint16_t)j : kTailOut;
                     val[t] = L.sval[e];
-                    mask |= 1u << tail_owner(blk, L.ncolours, j);
+                    if (in) mask |= 1u << tail_owner(blk, L.ncolours, j);
                 }
             }
             if (l > 0) {   // the row's value goes to its members, its right-hand side comes from them
@@ -482,9 +489,10 @@ __global__ void __launch_bounds__(kPackThreads) k_tail_pack(const TailDesc<T>* D
                 T* memw = reinterpret_cast<T*>(img + D.o_memw) + m0;
                 for (int k = kb; k < k1; ++k) {
                     const int m = F.ridx[k];
-                    mem[k - kb] = (uint16_t)m;
-                    if (kScaled) memw[k - kb] = F.t[m];
-                    mask |= 1u << tail_owner(D.blk + F.blk0, F.ncolours, m);
+                    const bool in = index_ok(m, F.n, D.err);
+                    mem[k - kb] = in ? (uint16_t)m : kTailOut;
+                    if (kScaled) memw[k - kb] = in ? F.t[m] : T(0);
+                    if (in) mask |= 1u << tail_owner(D.blk + F.blk0, F.ncolours, m);
                 }
                 o.members = (uint32_t)(k1 - kb);
             }
@@ -495,7 +503,10 @@ __global__ void __launch_bounds__(kPackThreads) k_tail_pack(const TailDesc<T>* D
         if (!coarsest) {
             reinterpret_cast<T*>(img + D.o_dinv)[gi] = has ? L.dinv[row] : T(0);
             const int g = has ? L.agg[row] : -1;
-            reinterpret_cast<uint16_t*>(img + D.o_agg)[gi] = g >= 0 ? (uint16_t)g : (uint16_t)0xffff;
+            const bool in = g < 0 || index_ok(g, L.nc, D.err);
+            reinterpret_cast<uint16_t*>(img + D.o_agg)[gi] = g < 0 ? (uint16_t)0xffff
+                                                             : in  ? (uint16_t)g
+                                                                   : kTailOut;
             if (kScaled) reinterpret_cast<T*>(img + D.o_aggw)[gi] = g >= 0 ? L.t[row] : T(0);
         }
     }
