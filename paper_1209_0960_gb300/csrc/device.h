@@ -246,6 +246,8 @@ struct DevLevel {
     int32_t lpr_wide = 0;             // lanes per row of launches over >= wide_rows rows
     int32_t wide_rows = 0x7fffffff;
     bool fused_restrict = false;      // residual and restriction in one kernel (lpr == 0)
+    bool late_restrict = false;       // the level above a dissected coarsest solve: the launch
+                                      // before the solve triggers it late
     bool fused_ok = false;            // the level allows the fused kernel (two colours,
                                       // aggregates of at most 32 rows of colour 1)
     int32_t* err = nullptr;           // device status word for kernel-side errors (timeouts)

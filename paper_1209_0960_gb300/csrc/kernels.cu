@@ -312,6 +312,17 @@ __host__ __device__ constexpr int unroll_of() { return LPR == 1 ? 24 : LPR == 2 
 // Late trigger against no overlap on wide grids, one iteration: layered
 // 192x160x145 float64 905 -> 837 us, anisotropic 256x224x209 mixed 1499 ->
 // 1457 us, log-normal 128^3 mixed 433 -> 421 us.
+//
+// The launches of the dissected coarsest solve and the one before it trigger
+// late whatever their grid.  Grids that all trigger at entry let the launch
+// after them start while they wait themselves, and so on down the stream: the
+// solve's blocks then sat on the SMs, with tens of KB of shared memory each,
+// under the passes of the level above, which took up to twice as long (V-cycle
+// from that level in float64: 16,089 rows 107.6 -> 76.5 us, 18,075 rows of a
+// neighbour graph 146 -> 82, 33,736 rows 119.5 -> 94.9, 19,522 rows of a 27-point
+// stencil 211 -> 157; float32 the same or up to 3 % less).  Late on every launch
+// gains as much there but loses elsewhere (64x64 PCG 1012 -> 1030 us, 128^3 mixed
+// 8.41 -> 8.54 ms, layered 35.1 -> 35.4 ms).
 __device__ __forceinline__ void trigger_early(const VArgs& a) {
     if (!a.late) pdl_launch_dependents();
 }
@@ -2309,7 +2320,7 @@ void vbatch_launch(const VRec* const* recs, int n, cudaStream_t s) {
         smem = std::max(smem, recs[k]->smem);
         if (recs[k]->carve != carve) carve = -1;
     }
-    for (int k = 0; k < n; ++k) p.a[k].late = p.bstart[n] > g_overlap_max_blocks;
+    for (int k = 0; k < n; ++k) p.a[k].late |= p.bstart[n] > g_overlap_max_blocks;
     // the 48 KB default covers static and dynamic shared memory together
     if (smem > kDefaultDynSmem) raise_dyn_smem(k_batched<Body>, smem);
     launch_kernel_carve(k_batched<Body>, p.bstart[n], recs[0]->block, smem, carve, true, s, p);
@@ -2339,7 +2350,7 @@ void vlaunch(int grid, int block, size_t smem, cudaStream_t s, const VArgs& a, i
     }
     if (smem > kDefaultDynSmem) raise_dyn_smem(k_single<Body>, smem);
     VArgs q = a;
-    q.late = grid > g_overlap_max_blocks;
+    q.late |= grid > g_overlap_max_blocks;
     launch_kernel_carve(k_single<Body>, grid, block, smem, carve, true, s, q);
 }
 
@@ -2503,6 +2514,7 @@ void residual_restrict_impl(const DevLevel& L, const T* b, const T* x, T* r, T* 
     a.dv = A.diag;
     a.b = b;
     a.x = const_cast<T*>(x);
+    a.late = L.fused_restrict && L.late_restrict;
     if (L.fused_restrict) {
         if (L.n > c1) {
             a.idx = L.agg;
@@ -2552,6 +2564,7 @@ void residual_restrict_impl(const DevLevel& L, const T* b, const T* x, T* r, T* 
     q.t = A.t;
     q.b = r;
     q.out = bc;
+    q.late = L.late_restrict;
     vlaunch<RestrictBody<T, SC>>(blocks_for(L.n_coarse), kBlock, 0, s, q);
 }
 
@@ -2703,6 +2716,7 @@ void dissected_impl(const DissDesc& D, const DissDesc* dev, const TB* b, TB* x, 
     a.dv = dev;
     a.b = b;
     a.x = x;
+    a.late = 1;   // see trigger_early
     const size_t smem = sizeof(double) * (size_t)(D.ns > 0 ? D.nI : D.longest);
     vlaunch<DissFirstBody<TB>>(D.nblk + (D.ns + kDissThreads / 32 - 1) / (kDissThreads / 32), kDissThreads,
                                smem, s, a);

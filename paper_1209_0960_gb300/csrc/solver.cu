@@ -1820,6 +1820,7 @@ void setup_impl(const amg_csr* A, const amg_params* prm, amg_ctx** out) {
     bool spd;
     if (!diss.order.empty()) {
         spd = dissect_device(c->hl[nlev - 1].A, diss, c->mem, c->diss, s);
+        if (nlev > 1) c->dl[nlev - 2].late_restrict = true;
     } else {
         c->Ainv = c->mem.alloc<double>((size_t)c->nL * c->nL);
         spd = dense_inverse_device(dA[nlev - 1], c->Ainv, s);
