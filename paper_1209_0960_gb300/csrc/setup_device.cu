@@ -621,17 +621,36 @@ void build_level_device(const DevCsr& A, const HostCsr& Ah, const std::vector<in
     }
     // lanes per row: the staged one-row-per-thread kernels on sparse rows
     // (bandwidth bound), several lanes on the denser coarse rows (gather
-    // latency bound).  Split levels read about half a row a pass, and the fewer
-    // rows a pass has, the more its time is one row's chain of loads, sums and
-    // instruction fetches.  Measured, V-cycle from the level, best shape against
-    // 4 lanes in blocks of 256: 6,619 rows 70.6 us (8 lanes, 128 threads) against
-    // 87.0; 8,204 rows 66.0 (8, 128) against 90.3; 51,913 rows 144.2 (4, 128)
-    // against 149.3; 77,212 rows 185.0 (2, 128) against 190.5; 610,622 rows
-    // 445.6 (1, 256) against 492.0; 1,671,533 rows 519.5 (1, 256) against 580.6.
+    // latency bound).  On a split level a pass reads about half a row, and the
+    // fewer rows it has, the more its time is one row's chain of loads, sums and
+    // instruction fetches, which more lanes shorten; the longer the rows, the
+    // further up that holds.  V-cycle from the level in float64, us, by lanes in
+    // blocks of 128 (256 with the same lanes: at most 2 % faster, up to 14 % slower):
+    //   rows       entries a row     8      4      2      1
+    //   8,268          11.4         60     66     74    111
+    //   16,187          6.0         57     57     60     74
+    //   34,032         15.5        108    118    129    199
+    //   49,278         15.6        154    163    171    237
+    //   51,932         11.7        144    141    148    189
+    //   76,393         14.9        186    180    192    257
+    //   105,089         8.6        193    165    164    198
+    //   128,547        11.8        222    186    185    220
+    //   259,103         7.6        281    249    234    229
+    //   269,587        11.9        313    291    269    295
+    //   314,662         6.4        307    251    245    227
+    //   391,841        11.9        410    355    346    352
+    //   612,615        10.9        546    447    422    414
+    //   1,661,243      10.9       1168    874    806    754
+    //   36,115         29.9        179    229    257    483
+    //   70,655         30.3        270    319    348    574
+    //   137,869        30.6        374    409    451    727
+    //   237,932        30.8        548    538    571    896
+    //   463,995        31.0        757    745    723    973
     const double avg = n > 0 ? (double)L.nnz_off / n : 0.0;
     if (split) {
-        L.lpr = n <= 20000 ? 8 : n <= 60000 ? 4 : n <= 300000 ? 2 : 1;
-        L.block = n <= 300000 ? 128 : 256;
+        if (avg > 16.0) L.lpr = n <= 200000 ? 8 : n <= 350000 ? 4 : 2;
+        else L.lpr = n <= 50000 ? 8 : n <= 100000 ? 4 : n <= (avg > 8.0 ? 450000 : 250000) ? 2 : 1;
+        L.block = 128;
     } else {
         L.lpr = (avg <= 7.0 && staged_fits(L)) ? 0 : avg <= 16.0 ? 4 : 8;
     }
