@@ -525,6 +525,12 @@ int amg_device_checks(void);
  * col < the level's rows). */
 int amg_debug_set_column(amg_ctx *c, int32_t l, int32_t row, int32_t k, int32_t col);
 
+/* Checked build only (AMG_EINVAL in the regular one): contexts that this thread
+ * sets up later see a device that holds clusters of at most `blocks` thread
+ * blocks (0 .. 16; 16 at first), to test that the kernels that run as larger
+ * clusters are then left to the ordinary launches.  Errors: AMG_EINVAL. */
+int amg_debug_cluster_limit(int32_t blocks);
+
 /* Thread-local description of the last error on this thread ("" if none). */
 const char *amg_last_error(void);
 

@@ -146,6 +146,7 @@ _SIGNATURES = {
     "amg_server_destroy": ([_c_vp], ctypes.c_int),
     "amg_last_error": ([], ctypes.c_char_p),
     "amg_device_checks": ([], ctypes.c_int),
+    "amg_debug_cluster_limit": ([_c_i32], ctypes.c_int),
     "amg_debug_set_column": ([_c_vp, _c_i32, _c_i32, _c_i32, _c_i32], ctypes.c_int),
 }
 

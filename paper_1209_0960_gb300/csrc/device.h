@@ -404,6 +404,11 @@ void raise_dyn_smem(void (*kernel)(KArgs...), size_t bytes) {
     raise_dyn_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 
+// How many clusters of `blocks` blocks of a kernel the current device can hold at
+// once, with `smem` bytes of dynamic shared memory a block; 0, and no error left
+// behind, where the runtime refuses the cluster or the question.
+int resident_clusters(const void* func, int blocks, int threads, size_t smem);
+
 // carve >= 0: the launch's preferred shared-memory carveout, in percent of
 // the SM's maximum shared memory (the rest of the unified L1/shared array is
 // L1 cache); -1: the driver's choice.  any_grid: the launch may overlap its
@@ -828,6 +833,11 @@ struct amg_ctx {
 };
 
 namespace amg {
+#ifdef AMG_DEVICE_CHECKS
+// largest cluster resident_clusters admits on this thread (amg_debug_cluster_limit)
+extern thread_local int t_cluster_limit;
+#endif
+
 // whether the levels from l0 down can run as a tail
 bool tail_fits(const amg_ctx* c, int l0, bool f32);
 // the tail from level l0, built on first use (not while a stream is captured)

@@ -21,6 +21,7 @@
 
 #include <map>
 #include <mutex>
+#include <tuple>
 
 #include "device.h"
 #include "device_util.cuh"
@@ -2226,6 +2227,51 @@ void raise_dyn_smem(const void* func, size_t bytes) {
     cur = bytes;
 }
 
+#ifdef AMG_DEVICE_CHECKS
+thread_local int t_cluster_limit = 16;
+#endif
+
+// The answers to the questions of one setup take about 0.1 ms of 17 (37x52x29),
+// so they are kept for the device, in steps of 16 KB of shared memory (asked for
+// the upper end).
+int resident_clusters(const void* func, int blocks, int threads, size_t smem) {
+#ifdef AMG_DEVICE_CHECKS
+    if (blocks > t_cluster_limit) return 0;
+#endif
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, int, size_t>, int> answers;
+    constexpr size_t kStep = 16 * 1024, kMost = 220 * 1024;
+    smem = std::max(smem, std::min((smem + kStep - 1) / kStep * kStep, kMost));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    try {
+        int dev = 0, clusters = 0;
+        AMG_CUDA_TRY(cudaGetDevice(&dev));
+        const auto key = std::make_tuple(dev, func, blocks, smem);
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = answers.find(key);
+        if (it != answers.end()) return it->second;
+        if (smem > 0) raise_dyn_smem(func, smem);
+        // more than 8 blocks are not portable
+        if (blocks > 8)
+            AMG_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        AMG_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, func, &cfg));
+        answers[key] = clusters;
+        return clusters;
+    } catch (const Error&) {
+        cudaGetLastError();
+        return 0;
+    }
+}
+
 thread_local bool t_launch_overlap = false;
 int g_overlap_max_blocks = 304;
 int g_reduction_blocks = 1216;
@@ -2820,44 +2866,30 @@ void launch_cg_update(int n, double* x, double* r, const double* p, const double
                                                        w.sc, cond);
 }
 
-namespace {
-
-template <int W>
-cudaLaunchConfig_t cg_cluster_config(cudaLaunchAttribute* attr, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCgBlocks);
-    cfg.blockDim = dim3(kCgThreads);
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kCgBlocks;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    AMG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_cg_cluster<W>),
-                                      cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    return cfg;
-}
-
-}  // namespace
-
 bool cg_cluster_fits(const DevLevel& L) {
     if (L.n > kCgClusterRows) return false;
     int clusters = 0;
-    cudaLaunchAttribute attr[2];
-    cudaError_t e = cudaSuccess;
     AMG_WIDTH_DISPATCH(L.width, {
-        const cudaLaunchConfig_t cfg = cg_cluster_config<W>(attr, nullptr);
-        e = cudaOccupancyMaxActiveClusters(&clusters, k_cg_cluster<W>, &cfg);
+        clusters = resident_clusters(reinterpret_cast<const void*>(&k_cg_cluster<W>), kCgBlocks, kCgThreads, 0);
     });
-    if (e != cudaSuccess) cudaGetLastError();
-    return e == cudaSuccess && clusters > 0;
+    return clusters > 0;
 }
 
 void launch_cg_cluster(const DevLevel& L, double* r, const double* z, double* zold, double* p, double* q,
                        double* x, CgWork& w, LoopCond cond, cudaStream_t s) {
     AMG_WIDTH_DISPATCH(L.width, {
         cudaLaunchAttribute attr[2];
-        cudaLaunchConfig_t cfg = cg_cluster_config<W>(attr, s);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kCgBlocks);
+        cfg.blockDim = dim3(kCgThreads);
+        cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kCgBlocks;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        AMG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void*>(&k_cg_cluster<W>),
+                                          cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         if (t_launch_overlap) {
             attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[1].val.programmaticStreamSerializationAllowed = 1;

@@ -2300,6 +2300,18 @@ int amg_device_checks(void) {
 #endif
 }
 
+int amg_debug_cluster_limit(int32_t blocks) {
+    return Guard::run([&] {
+#ifndef AMG_DEVICE_CHECKS
+        (void)blocks;
+        throw Error{AMG_EINVAL, "amg_debug_cluster_limit exists in the checked build only"};
+#else
+        if (blocks < 0 || blocks > 16) throw Error{AMG_EINVAL, "blocks must be 0 .. 16"};
+        t_cluster_limit = blocks;
+#endif
+    });
+}
+
 int amg_debug_set_column(amg_ctx* c, int32_t l, int32_t row, int32_t k, int32_t col) {
     return Guard::run([&] {
 #ifndef AMG_DEVICE_CHECKS

@@ -703,7 +703,14 @@ struct TailPlan {
 // the float64 rate, so a solve of many rows is a launch over all SMs.
 inline bool tail_dense(int32_t nL) { return nL <= 256; }
 
-// Blocks of the cluster for the tail from level l0; 0 if it does not fit.
+template <typename T>
+const void* tail_kernel(int nc) {
+    void (*k)(const TailBatch) = nc == 1 ? &k_tail<T, 1> : nc == 8 ? &k_tail<T, 8> : &k_tail<T, 16>;
+    return reinterpret_cast<const void*>(k);
+}
+
+// Blocks of the cluster for the tail from level l0; 0 if it does not fit: in
+// shared memory, or on a device (or a part of one) that cannot hold the cluster.
 template <typename T>
 int tail_cluster(const amg_ctx* c, int l0, bool m32) {
     const int nlev = (int)c->dl.size(), m = nlev - 1 - l0;
@@ -718,8 +725,9 @@ int tail_cluster(const amg_ctx* c, int l0, bool m32) {
     const bool one = tail_dense(c->nL);
     for (int nc : {1, 8, 16}) {
         if (nc < tail_blocks(c->dl[l0].n)) continue;
-        if (TailPlan<T>(c->dl, l0, nc, true, one, m32).smem <= kTailSmem &&
-            (one || TailPlan<T>(c->dl, l0, nc, false, true, m32).smem <= kTailSmem))
+        int64_t smem = TailPlan<T>(c->dl, l0, nc, true, one, m32).smem;
+        if (!one) smem = std::max(smem, TailPlan<T>(c->dl, l0, nc, false, true, m32).smem);
+        if (smem <= kTailSmem && resident_clusters(tail_kernel<T>(nc), nc, kTailThreads, (size_t)smem) > 0)
             return nc;
     }
     return 0;
