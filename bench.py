@@ -147,9 +147,10 @@ def parse_args():
     ap.add_argument("--lanes-per-row", type=str, default="", metavar="L0,L1,...",
                     help="fixed launch shapes per level instead of tuning (0 = staged "
                          "kernels, else 1/2/4/8 lanes per row, with a suffix h for blocks of "
-                         "128 threads and s for one dependency-driven kernel per smoothing "
-                         "sweep; staged levels may add cP for a shared-memory carveout of P "
-                         "percent, e.g. 0,0c58,2h,4hs), for reproducible profiles")
+                         "128 threads, s for one dependency-driven kernel per smoothing "
+                         "sweep and t for the cluster launch of the small levels; staged levels "
+                         "may add cP for a shared-memory carveout of P percent, e.g. "
+                         "0,0c58,2h,4hs,8ht), for reproducible profiles")
     ap.add_argument("--aggregation-device", type=int, choices=[0, 1], default=0,
                     help="with --aggregation-tile: run the tiles on the GPU (1) or on host threads")
     args = ap.parse_args()
@@ -406,13 +407,15 @@ def parse_lanes(text: str) -> list:
     out = []
     for v in (v.strip() for v in text.split(",")):
         if v:
-            m = re.fullmatch(r"(\d+)(h?)(s?)(?:c(\d+))?", v)
+            m = re.fullmatch(r"(\d+)(h?)(s?)(t?)(?:c(\d+))?", v)
             if not m:
                 raise ValueError(f"--lanes-per-row: cannot read {v!r}")
             lanes = int(m.group(1))
             if m.group(3):
                 lanes |= 0x100   # AMG_SHAPE_SWEEP: one dependency-driven kernel per sweep
-            carve = int(m.group(4)) if m.group(4) else None
+            if m.group(4):
+                lanes |= 0x200   # AMG_SHAPE_CLUSTER: in the launch of the small levels
+            carve = int(m.group(5)) if m.group(5) else None
             out.append((lanes, 128 if m.group(2) else 0, carve))
     return out
 
@@ -430,6 +433,7 @@ def shape_string(levels):
     for lv in levels[:-1]:
         v = str(lv["lanes_per_row"]) + ("h" if lv["threads_per_block"] == 128 else "")
         v += "s" if lv["sweep"] else ""
+        v += "t" if lv.get("cluster") else ""
         v += f"c{lv['carveout']}" if lv["carveout"] >= 0 else ""
         out.append(v)
     return ",".join(out)

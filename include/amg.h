@@ -75,6 +75,11 @@ extern "C" {
  * dependency-driven kernel instead of one launch per colour pass */
 #define AMG_SHAPE_SWEEP 0x100
 
+/* or'ed into amg_set_level_shape's lanes_per_row: the level runs in the cluster
+ * launch of the small levels whenever every level below it does and they fit;
+ * the lanes and block size are its shape otherwise */
+#define AMG_SHAPE_CLUSTER 0x200
+
 typedef struct amg_ctx amg_ctx;
 
 typedef struct {
@@ -187,6 +192,10 @@ typedef struct {
                                  percent of the SM's maximum shared memory (the rest of the
                                  unified L1/shared array caches the neighbour gathers);
                                  -1: the driver's choice */
+    int32_t cluster;          /* 1: the level runs in the cluster launch of the small levels
+                                 (one launch for their part of the V-cycle, or two around
+                                 the coarsest solve); the shape above then applies to
+                                 launches of its own only */
 } amg_level_info;
 
 typedef struct {
@@ -351,13 +360,17 @@ int amg_export_level(const amg_ctx *c, int32_t l, int32_t *row_ptr, int32_t *col
  * two-colour levels with the fused residual): each smoothing sweep then runs
  * as one kernel whose blocks wait, with bounded polls, only for the earlier
  * colour-pass blocks they depend on (planned on the host from the level's
- * graph at the first use of a block size).  threads_per_block: 256 or 128 for
+ * graph at the first use of a block size), or with AMG_SHAPE_CLUSTER (levels
+ * of three or more colours).  Without that flag the level runs as launches of its
+ * own: it leaves the cluster launch of the small levels, and so do the levels
+ * above it.  threads_per_block: 256 or 128 for
  * lanes_per_row >= 1 (0 means 256; the staged kernels always use 256).
  * Results differ only in the order of floating-point sums (a sweep gives the
  * same values as the pass-per-launch kernels of its lanes and block size).
  * The CUDA graphs of the context are rebuilt on the next solve.  Errors:
  * AMG_EINVAL (l, lanes_per_row or threads_per_block out of range, 0 lanes on a
- * level whose tile does not fit, a sweep where it is not allowed). */
+ * level whose tile does not fit, a sweep or the cluster where it is not
+ * allowed). */
 int amg_set_level_shape(amg_ctx *c, int32_t l, int32_t lanes_per_row, int32_t threads_per_block);
 
 /* Preferred shared-memory carveout of level l's staged kernels (the level's
@@ -518,9 +531,8 @@ int amg_device_checks(void);
 /* Checked build only (AMG_EINVAL in the regular one): overwrite the column
  * index of the k-th stored off-diagonal entry of row `row` (level-l
  * numbering; l >= 1) with `col` on the device, to test that the checks catch
- * a corrupt hierarchy.  A column >= the level's rows is never dereferenced by
- * any kernel of either build (neighbours at positions beyond the pass bound
- * are skipped), so this cannot make a kernel read out of range.  The context
+ * a corrupt hierarchy.  A column >= the level's rows is reported by every
+ * kernel of this build that meets it and never used as an index.  The context
  * is corrupt afterwards: free it.  Errors: AMG_EINVAL (build, l, row, k, or
  * col < the level's rows). */
 int amg_debug_set_column(amg_ctx *c, int32_t l, int32_t row, int32_t k, int32_t col);

@@ -35,6 +35,7 @@ _SOLVE_STATUSES = (AMG_ENOTCONV, AMG_ENOTSPD, AMG_ENONFINITE, AMG_ERANGE, AMG_ET
 AMG_FP64 = 0
 AMG_FP32_IN_FP64 = 1
 AMG_SHAPE_SWEEP = 0x100   # or'ed into lanes_per_row: one dependency-driven kernel per sweep
+AMG_SHAPE_CLUSTER = 0x200   # or'ed into lanes_per_row: in the cluster launch of the small levels
 
 _c_i32 = ctypes.c_int32
 _c_dbl = ctypes.c_double
@@ -67,7 +68,8 @@ class amg_level_info(ctypes.Structure):
                 ("max_agg_size", _c_i32), ("n_isolated", _c_i32), ("n_dirichlet", _c_i32),
                 ("vcycle_bytes_fp64", _c_dbl), ("vcycle_bytes_fp32", _c_dbl),
                 ("lanes_per_row", _c_i32), ("threads_per_block", _c_i32), ("sweep", _c_i32),
-                ("compact", _c_i32), ("staged_entries", ctypes.c_int64), ("carveout", _c_i32)]
+                ("compact", _c_i32), ("staged_entries", ctypes.c_int64), ("carveout", _c_i32),
+                ("cluster", _c_i32)]
 
 
 class amg_summary(ctypes.Structure):

@@ -181,6 +181,21 @@ double level_vcycle_bytes(const DevLevel& L, int vb) {
     return t;
 }
 
+// The launch shapes the levels run now (after find_tail: a level's shape decides
+// about the cluster for those above it too).
+void fill_shapes(amg_ctx* c) {
+    const int last = (int)c->linfo.size() - 1;
+    for (int l = 0; l <= last; ++l) {
+        amg_level_info& li = c->linfo[l];
+        const DevLevel& d = c->dl[l];
+        li.lanes_per_row = l < last ? d.lpr : 0;
+        li.threads_per_block = l < last ? d.block : 0;
+        li.sweep = (l < last && d.sweep) ? 1 : 0;
+        li.carveout = l < last ? d.carve : -1;
+        li.cluster = (l < last && l >= c->tail_l0) ? 1 : 0;
+    }
+}
+
 void fill_info(amg_ctx* c) {
     const int L = (int)c->dl.size();
     c->linfo.assign(L, amg_level_info{});
@@ -199,10 +214,6 @@ void fill_info(amg_ctx* c) {
         li.n_dirichlet = last ? 0 : h.agg.n_dirichlet;
         li.vcycle_bytes_fp64 = last ? coarsest_bytes(c, 8) : level_vcycle_bytes(d, 8);
         li.vcycle_bytes_fp32 = last ? coarsest_bytes(c, 4) : level_vcycle_bytes(d, 4);
-        li.lanes_per_row = last ? 0 : d.lpr;
-        li.threads_per_block = last ? 0 : d.block;
-        li.sweep = (!last && d.sweep) ? 1 : 0;
-        li.carveout = last ? -1 : d.carve;
         li.compact = d.soff ? 1 : 0;
         li.staged_entries = d.soff ? d.stage_entries : d.padded;
         b64 += li.vcycle_bytes_fp64;
@@ -210,6 +221,7 @@ void fill_info(amg_ctx* c) {
         if (l == 0) nnz0 = li.nnz;
         nnzs += li.nnz;
     }
+    fill_shapes(c);
     c->summary.num_levels = L;
     c->summary.coarsest_n = c->nL;
     c->summary.operator_complexity = nnzs / nnz0;
@@ -1973,12 +1985,7 @@ int amg_set_precision(amg_ctx* c, int32_t precision, int32_t flexible_cg) {
             c->summary.autotune_ms += autotune_shapes(c);
         }
         apply_shapes(c);
-        for (int l = 0; l + 1 < (int)c->dl.size(); ++l) {
-            c->linfo[l].lanes_per_row = c->dl[l].lpr;
-            c->linfo[l].threads_per_block = c->dl[l].block;
-            c->linfo[l].sweep = c->dl[l].sweep ? 1 : 0;
-            c->linfo[l].carveout = c->dl[l].carve;
-        }
+        fill_shapes(c);
         leave(c);
     });
 }
@@ -2157,23 +2164,23 @@ int amg_set_level_shape(amg_ctx* c, int32_t l, int32_t lanes_per_row, int32_t th
         if (threads_per_block != 0 && threads_per_block != 256 && threads_per_block != 128)
             throw Error{AMG_EINVAL, "threads_per_block must be 0, 256 or 128"};
         const bool sweep = (lanes_per_row & AMG_SHAPE_SWEEP) != 0;
-        const int lanes = lanes_per_row & ~AMG_SHAPE_SWEEP;
-        const int code = lanes | (threads_per_block == 128 ? kHalfBlock : 0) | (sweep ? kSweep : 0);
+        const bool cluster = (lanes_per_row & AMG_SHAPE_CLUSTER) != 0;
+        const int lanes = lanes_per_row & ~(AMG_SHAPE_SWEEP | AMG_SHAPE_CLUSTER);
+        const int code = lanes | (threads_per_block == 128 ? kHalfBlock : 0) | (sweep ? kSweep : 0) |
+                         (cluster ? kTail : 0);
         if (lanes < 0 || lanes > 8 || !shape_allowed(c->dl[l], code))
             throw Error{AMG_EINVAL, "lanes_per_row must be 1, 2, 4 or 8 (optionally with "
                                     "AMG_SHAPE_SWEEP on a level of at most 2^20 rows that is not "
                                     "two-colour fused), or 0 (256 threads) on a level whose staged "
-                                    "tile fits in 96 KB"};
+                                    "tile fits in 96 KB; AMG_SHAPE_CLUSTER on levels of three or "
+                                    "more colours, without AMG_SHAPE_SWEEP"};
         enter(c);
         AMG_CUDA_TRY(cudaStreamSynchronize(c->stream));   // no graph of this context in flight
         drop_graphs(c);
         set_shape(c, l, code);
         find_tail(c);
         c->shapes[c->precision][l] = code;
-        c->linfo[l].lanes_per_row = c->dl[l].lpr;
-        c->linfo[l].threads_per_block = c->dl[l].block;
-        c->linfo[l].sweep = c->dl[l].sweep ? 1 : 0;
-        c->linfo[l].carveout = c->dl[l].carve;
+        fill_shapes(c);
         leave(c);
     });
 }
@@ -2193,7 +2200,7 @@ int amg_set_level_carveout(amg_ctx* c, int32_t l, int32_t percent) {
         set_shape(c, l, code);
         find_tail(c);
         c->shapes[c->precision][l] = code;
-        c->linfo[l].carveout = c->dl[l].carve;
+        fill_shapes(c);
         leave(c);
     });
 }
