@@ -143,8 +143,10 @@ typedef struct {
                                  V-cycle from that level, replayed as a CUDA graph in the
                                  context's precision) and keeps the fastest; choices are
                                  cached per process by level signature (precision, size
-                                 class, slice width, mean row length, colours), so later
-                                 setups of similar levels reuse them.  Shapes change the
+                                 class, slice width, mean row length, colours; and for
+                                 the cluster launch of the small levels, whether it
+                                 holds the coarsest solve), so later setups of similar
+                                 levels reuse them.  Shapes change the
                                  order of floating-point sums only. */
 } amg_params;
 

@@ -306,6 +306,8 @@ struct DevLevel {
 // rows of a level of the tail (tail.cu) stay below this: its columns have 16
 // bits, and this value marks none
 constexpr int32_t kTailMaxRows = 65535;
+// rows of the largest coarsest level that is solved inside the tail's launch
+constexpr int32_t kTailDenseMax = 256;
 
 // largest tile of the staged kernels (index and value of the entries of 8
 // consecutive slices): two blocks still fit on an SM.  With the common width

@@ -824,8 +824,26 @@ ShapeKey shape_key(const amg_ctx* c, int l) {
     return {c->precision, size_class, (L.width + 3) / 4, mean, L.ncolours, l == 0 ? 1 : 0};
 }
 
+// What the tail is to level l with the shapes of the levels below it.
+enum TailCase { kTailClosed = 0, kTailOutside = 1, kTailInside = 2 };   // the coarsest solve's place
+TailCase tail_case(const amg_ctx* c, int l) {
+    if (!c->dl[l].split || !(l == (int)c->dl.size() - 2 || c->tail_l0 <= l + 1) ||
+        !tail_fits(c, l, c->precision == AMG_FP32_IN_FP64))
+        return kTailClosed;
+    return c->nL <= kTailDenseMax ? kTailInside : kTailOutside;
+}
+
+// A tuned level: its shape as launches of its own, and whether the tail was
+// faster where it was open (-1: not timed yet).  The two are kept apart because
+// hierarchies that agree on the level differ in what is below it.
+struct TunedShape {
+    int own = 0;
+    int tail[3] = {0, -1, -1};
+    int code(TailCase t) const { return own | (t != kTailClosed && tail[t] > 0 ? kTail : 0); }
+};
+
 std::mutex g_shape_mu;
-std::map<ShapeKey, int> g_shape_cache;
+std::map<ShapeKey, TunedShape> g_shape_cache;
 
 // Device time of one replay of the V-cycle from level l (the whole
 // preconditioner for l = 0), as a CUDA graph: the minimum over three batches
@@ -884,51 +902,71 @@ double autotune_shapes(amg_ctx* c) {
     for (int l = nlev - 2; l >= 0; --l) {
         DevLevel& L = c->dl[l];
         const ShapeKey key = shape_key(c, l);
+        const TailCase tc = tail_case(c, l);
+        const int rule = shape_of(L), rule_own = rule & ~kTail;
+        TunedShape tuned;
+        bool own_known = false;
         {
             std::lock_guard<std::mutex> lk(g_shape_mu);
             auto it = g_shape_cache.find(key);
-            if (it != g_shape_cache.end() && shape_allowed(L, it->second)) {
-                set_shape(c, l, it->second);
-                find_tail(c);
-                continue;
+            if (it != g_shape_cache.end() && shape_allowed(L, it->second.own)) {
+                tuned = it->second;
+                own_known = true;
             }
+        }
+        const bool tail_known = tc == kTailClosed || tuned.tail[tc] >= 0;
+        if (own_known && tail_known) {
+            set_shape(c, l, tuned.code(tc));
+            find_tail(c);
+            continue;
         }
         if (!timed) {
             zero_inputs();
             timed = true;
         }
-        const int rule = shape_of(L);
-        double t_rule = 1e30, t_best = 1e30;
-        int best = rule;
-        std::vector<int> tries = {kStaged, 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4, 4 | kHalfBlock, 8,
-                                  8 | kHalfBlock, 2 | kSweep, 2 | kHalfBlock | kSweep, 4 | kSweep,
-                                  4 | kHalfBlock | kSweep, 8 | kSweep, 8 | kHalfBlock | kSweep};
-        // staged kernels also with a smaller shared-memory carveout (percent
-        // of the maximum 228 KB: 100, 132 or 164 KB), leaving more L1 for the
-        // neighbour gathers
-        if (uses_shared_memory(L))
-            for (int pct : {44, 58, 72}) tries.push_back(with_carve(kStaged, pct));
-        // the tail, where every level below is in it
-        if (L.split && (l == nlev - 2 || c->tail_l0 <= l + 1) &&
-            tail_fits(c, l, c->precision == AMG_FP32_IN_FP64))
-            tries.push_back(rule | kTail);
-        for (int lanes : tries) {
-            if (!shape_allowed(L, lanes)) continue;
-            set_shape(c, l, lanes);
+        auto time_shape = [&](int code) {
+            set_shape(c, l, code);
             find_tail(c);
-            const double t = time_vcycle_from(c, l);
-            if (lanes == rule) t_rule = t;
-            if (t < t_best) {
-                t_best = t;
-                best = lanes;
+            return time_vcycle_from(c, l);
+        };
+        double t_own = 1e30;
+        if (own_known) {
+            t_own = time_shape(tuned.own);
+        } else {
+            std::vector<int> tries = {kStaged, 1, 1 | kHalfBlock, 2, 2 | kHalfBlock, 4, 4 | kHalfBlock, 8,
+                                      8 | kHalfBlock, 2 | kSweep, 2 | kHalfBlock | kSweep, 4 | kSweep,
+                                      4 | kHalfBlock | kSweep, 8 | kSweep, 8 | kHalfBlock | kSweep};
+            // staged kernels also with a smaller shared-memory carveout (percent
+            // of the maximum 228 KB: 100, 132 or 164 KB), leaving more L1 for the
+            // neighbour gathers
+            if (uses_shared_memory(L))
+                for (int pct : {44, 58, 72}) tries.push_back(with_carve(kStaged, pct));
+            double t_rule = 1e30;
+            tuned.own = rule_own;
+            for (int code : tries) {
+                if (!shape_allowed(L, code)) continue;
+                const double t = time_shape(code);
+                if (code == rule_own) t_rule = t;
+                if (t < t_own) {
+                    t_own = t;
+                    tuned.own = code;
+                }
+            }
+            if (t_rule <= 1.03 * t_own) {
+                tuned.own = rule_own;
+                t_own = t_rule;
             }
         }
-        if (t_rule <= 1.03 * t_best) best = rule;
+        if (tc != kTailClosed && !tail_known) {
+            const double t = time_shape(tuned.own | kTail);
+            tuned.tail[tc] = ((rule & kTail) ? t <= 1.03 * t_own : 1.03 * t < t_own) ? 1 : 0;
+        }
         // a context tuning the same signature concurrently may have stored
         // its choice first: every context then runs the stored one
         std::lock_guard<std::mutex> lk(g_shape_mu);
-        const int stored = g_shape_cache.emplace(key, best).first->second;
-        set_shape(c, l, shape_allowed(L, stored) ? stored : best);
+        TunedShape& stored = g_shape_cache.emplace(key, tuned).first->second;
+        if (tc != kTailClosed && stored.tail[tc] < 0) stored.tail[tc] = tuned.tail[tc];
+        set_shape(c, l, (shape_allowed(L, stored.own) ? stored : tuned).code(tc));
         find_tail(c);
     }
     for (int l = 0; l + 1 < nlev; ++l) c->shapes[c->precision][l] = shape_of(c->dl[l]);

@@ -701,7 +701,7 @@ struct TailPlan {
 
 // Whether the coarsest solve joins the cluster's launch: 16 SMs have a tenth of
 // the float64 rate, so a solve of many rows is a launch over all SMs.
-inline bool tail_dense(int32_t nL) { return nL <= 256; }
+inline bool tail_dense(int32_t nL) { return nL <= kTailDenseMax; }
 
 template <typename T>
 const void* tail_kernel(int nc) {
