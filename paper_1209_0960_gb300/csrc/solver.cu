@@ -758,12 +758,26 @@ void plan_sweep(amg_ctx* c, int l, int rows, bool pre, SweepPlan& P) {
     AMG_CUDA_TRY(cudaStreamSynchronize(s));   // the host vectors go out of scope
 }
 
-// Levels that join the tail without being timed: in float64, where 16 SMs run
-// the arithmetic of a pass at a tenth of the device's rate, up to about 7,000
-// rows (6,619 rows: 69.8 us from the level against 73.8 as launches; 13,113
-// rows: 132 against 75 before the entries moved to shared memory); in float32
-// as far as the tail fits in shared memory (about 18,000 rows).
-inline bool tail_rule(const DevLevel& L, bool f32) { return L.split && (f32 || L.n <= 7000); }
+// Levels that join the tail without being timed: up to 7,000 rows, above which
+// the 16 SMs take longer over a pass than a launch over all of them does; in
+// float32 also larger levels of more than 16 entries a row, as far as they fit in
+// shared memory, whose launches are longer.  V-cycle from the level, us, tail
+// against launches of eight lanes:
+//   rows (entries a row)   float64       float32
+//   6,036  (11.3)        61.1   61.8   51.8   51.5
+//   6,641  (15.0)        71.6   73.7   57.4   63.4
+//   7,280   (5.8)        49.5   50.7   50.9   42.9
+//   7,852   (9.4)        63.6   59.8   61.4   51.6
+//   8,063  (14.2)        77.7   80.2   69.8   67.7
+//   8,257   (5.9)        61.7   53.4   59.9   48.1
+//   11,795 (11.5)           -   71.2   71.8   57.8
+//   18,075 (11.9)           -   83.4  105.1   73.5
+//   5,455  (16.4)        75.7   79.9   57.4   81.8
+//   7,218  (21.3)        88.1   94.0   65.9   79.6
+//   8,835  (28.7)           -    129   88.5  123.9
+inline bool tail_rule(const DevLevel& L, bool f32) {
+    return L.split && (L.n <= 7000 || (f32 && L.nnz_off > 16 * (int64_t)L.n));
+}
 
 // The first level of the tail under the levels' current shapes, and its
 // descriptors (built here: V-cycles are captured into graphs).  Called after
