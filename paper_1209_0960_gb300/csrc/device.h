@@ -387,9 +387,6 @@ struct CgWork {
 // matrices and index lists fixed at setup, so the overlap hides launch
 // latency and the first dependent loads of each kernel.  Set per calling
 // thread from the context at API entry.
-// Sets the condition of the device-side CG loop (a WHILE graph node) to
-// "not converged, no breakdown, fewer than maxit iterations" from the device
-// scalars; it also counts its own evaluations and stops at maxit.
 extern thread_local bool t_launch_overlap;
 // grids above this many blocks: CG kernels launch without the overlap (a wide
 // grid that starts early only occupies the SMs its predecessor is still

@@ -1677,9 +1677,18 @@ void init_device_pool(int device) {
 }
 
 // The dissection of the coarsest matrix where its solve reads less than half of
-// the whole inverse (empty: the dense inverse).  Below 2,000 rows the dense
-// product is a few microseconds and three launches would cost as much; the
-// float32 copy of coarsest_fp32 stays the dense inverse.
+// the whole inverse (empty: the dense inverse).  Solve and setup of the dense
+// inverse against the dissected one, float64, by rows of the coarsest level:
+//   2,089   14.3 us, 20 ms   20.4 us,  8 ms
+//   2,344   16.7 us, 25 ms   22.1 us,  9 ms
+//   2,561   22.5 us, 31 ms   18.6 us,  9 ms   (9-point)
+//   2,867   25.0 us, 36 ms   26.7 us, 14 ms   (27-point)
+//   3,250   26.9 us, 47 ms   22.5 us, 12 ms
+//   4,325   45.4 us          30.7 us
+// So from 2,600 rows on it is the faster solve; between that and 2,000 it costs 4
+// to 8 us a V-cycle and saves 12 ms or more of setup, which takes over a thousand
+// V-cycles to lose; below 2,000 that shrinks too.  The float32 copy of
+// coarsest_fp32 stays the dense inverse.
 Dissection coarsest_dissection(const HostCsr& A, const amg_params& p) {
     Dissection none;
     if (A.n < 2000 || p.coarsest_fp32) return none;
