@@ -44,7 +44,7 @@ def walk(tmp_path_factory):
     d = tmp_path_factory.mktemp("tiles")
     (d / "walk.cpp").write_text(SRC)
     subprocess.run([cxx, "-O1", "-std=c++17", "-fsanitize=signed-integer-overflow",
-                    "-fno-sanitize-recover", "-I", os.path.join(ROOT, "paper_1209_0960_gb300", "csrc"),
+                    "-fsanitize-undefined-trap-on-error", "-I", os.path.join(ROOT, "paper_1209_0960_gb300", "csrc"),
                     str(d / "walk.cpp"), "-o", str(d / "walk")], check=True, capture_output=True)
 
     def run(e, length):
